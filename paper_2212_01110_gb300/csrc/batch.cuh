@@ -56,19 +56,17 @@ void launch_node_ops_b(int which, const BInst<S>* bi, const BMap& m, int nblocks
 // for nx + nu.
 template <typename S>
 void launch_riccati_b(int which, const BInst<S>* bi, const BMap& m, int nblocks, int SL, cudaStream_t st);
-// riccati_tma.cu: the same passes with the staged (bulk-copy) kernels: chain
-// blocks of wpb warps, one block per node for the stages.
-struct TmaBatchShape {
-  uint32_t slot_bwd = 0, slot_fwd = 0;   // bytes of shared memory per chain warp
-  int wpb_bwd = 1, wpb_fwd = 1;          // warps per chain block
-  int nw_stage_bwd = 1, nw_stage_fwd = 1;  // warps per stage block
-  uint32_t smem_stage_bwd = 0, smem_stage_fwd = 0;
+// riccati_seq.cu: the same passes with the staged kernels, one block per node
+// sequence (stage -1 of a map: the chain region).
+struct SeqBatchShape {
+  int T = 32;                               // threads per block
+  uint32_t bytes_bwd = 0, bytes_fwd = 0;    // shared memory of a block
 };
 template <typename S>
-bool tma_batch_shape(const std::vector<KP<S>>& kps, int max_children, TmaBatchShape& sh);
+bool seq_batch_shape(const std::vector<KP<S>>& kps, SeqBatchShape& sh);
 template <typename S>
-void launch_riccati_tma_b(int which, const BInst<S>* bi, const BMap& m, int nblocks, int SL, const TmaBatchShape& sh,
-                          cudaStream_t st);
+void launch_seq_b(int which, const BInst<S>* bi, const BMap& m, int nblocks, const SeqBatchShape& sh,
+                  cudaStream_t st);
 // cta.cu: whole solves, one 128-thread block per instance (instances with
 // nx + nu <= max_nxu <= 62, Anderson memory 0, 3 or 5), at most max_rounds
 // rounds each; trace (or NULL) for a single instance.

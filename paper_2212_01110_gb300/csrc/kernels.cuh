@@ -11,7 +11,13 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "fxp.cuh"
+
 namespace spock {
+
+// bytes, rounded up to a multiple of 16 or 128
+__host__ __device__ inline uint32_t up16(uint32_t b) { return (b + 15u) & ~15u; }
+__host__ __device__ inline uint32_t up128(uint32_t b) { return (b + 127u) & ~127u; }
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kWarpsPerBlock = 4;        // 128-thread blocks for the warp-per-node kernels
@@ -114,6 +120,20 @@ struct KP {
   const S* __restrict__ Gf;
   const S* __restrict__ NB;
   const S* __restrict__ Kt;
+  // the factors as the sequence kernels read them (riccati_seq.cu), per matrix
+  // one 16-byte aligned block of gbB, gfB, nbB, ktB bytes, row-major:
+  //   pGb  [B | Abar] (nx x (nu + nx)),  pGf  [Abar | B]^T ((nx + nu) x nx),
+  //   pNB  [Rtilde^-1 | E] (nu x (nu + nx)) and K (nu x nx), E = Rtilde^-1 (K + W^T),
+  //   pKt  K^T (nx x nu).
+  // FP32: numbers.  FP64: fixed-point entries (fxp.cuh) followed by one exponent
+  // per column (pNB: per column of the first matrix, E's also for K's).
+  const unsigned char* __restrict__ pGb;
+  const unsigned char* __restrict__ pGf;
+  const unsigned char* __restrict__ pNB;
+  const unsigned char* __restrict__ pKt;
+  uint32_t gbB, gfB, nbB, ktB;
+  S* __restrict__ hb;   // [n - 1][hst] [B^c | Abar^c]^T q^c of the nonroot nodes
+  int32_t hst;
   const S* __restrict__ qs;
   const S* __restrict__ rs;
   const S* __restrict__ qns;

@@ -1,0 +1,608 @@
+// Riccati passes (Algorithm 2), a block per node sequence, every node's
+// factors staged in shared memory.
+//
+// A sequence is a run of nodes that follow one another through single
+// children: the chain below the last branching stage with its leaf (one launch
+// for all chains), or one node of a branching stage (one launch per stage).
+// The backward step of node k
+//   h   = sum over the children of h^c           (leaf: q^k = -xbar^k)
+//   g   = ubar^k - h_u
+//   d^k = Rt^-1 g,   q^k = h_x - xbar^k + E^T g - K^T ubar^k
+//   h^k = [Abar^k | B^k]^T q^k                   (not at the root)
+// with E = Rt^-1 (K + W^T), formed once with the factors (q^k = h_x - xbar^k +
+// K^T (d^k - ubar^k) + W d^k, so that d^k and q^k come from one product), reads
+// the factors of node k only and hands nx + nu numbers on to the parent: in
+// registers along a sequence, through p.hb between launches.  A branching
+// stage reads a quarter of what a step over the children's [Abar | B] reads at
+// four children per node; those of the chains' tops are streamed by the chain
+// launch.  The forward step of a node k > 0
+//   x^k = [Abar^k | B^k] (x; d)^parent,   u^parent = K^parent x^parent + d^parent
+// (u by the first child) is one product as well.
+//
+// T threads of a block work on one node at a time: thread (row group, column)
+// of a product, the row groups' partial sums added through shared memory.  One
+// more warp fetches the nodes' blocks by bulk asynchronous copies into a ring
+// of D slots (address arithmetic, fence and copies in one of the T threads
+// would lengthen every step, and so would a second barrier to wait on: 200
+// cycles each, measured).  What latency is left, and the serial sums and
+// barriers of a step, is covered by the other blocks of the SM.  FP64 products
+// are the exact integer sums of fxp.cuh.
+//
+// What bounds it and what it measured (GB300, nx = 50, nu = 20).  Chains of the
+// 62,805-node tree, FP64: backward 670 us (2.84 GB, 4.2 TB/s), forward 473 us
+// (2.2 GB), where direct-load kernels on the FP64 pipe took 1,073 and 705 us;
+// the FP32 chains of 4,096 sequences of five nodes run at 5.2 - 5.6 TB/s.  A
+// step alone takes 3.5 (backward) and 2.1 us (forward) in FP64, against 15.9
+// and 4.3, and 1.3 and 0.9 us in FP32, against 2.7 and 1.8.  The FP64 chains
+// are bound by the steps of the four resident blocks (about 28 cycles a row of
+// five wide multiply-adds and two shared loads, and 1,000 instructions of
+// conversions and barriers), the FP32 ones by memory latency.
+//
+// Bounded waits: a wait that exceeds kWaitLimit polls sets *p.err and the
+// thread stops waiting (the fetching warp: stops issuing); the block finishes
+// its loop on whatever the buffers hold (every access stays inside them), and
+// the fetching warp waits for its copies in flight (bounded) before it returns.
+#include <algorithm>
+#include <atomic>
+#include <vector>
+
+#include "batch.cuh"
+#include "kernels.cuh"
+#include "spock_internal.h"
+#include "tma.cuh"
+
+namespace spock {
+
+constexpr int kMaxSeqThreads = 256;   // T; 32 more fetch
+constexpr int kMaxSlots = 8;
+
+
+// Shared memory of a block, in bytes: D slots of one node's blocks each,
+// prepared vectors, partial sums.
+struct SeqLayout {
+  uint32_t item, vecA, vecB, part;
+  __host__ __device__ uint32_t bytes(int D) const { return D * item + vecA + vecB + part; }
+};
+__host__ __device__ inline int up4(int n) { return (n + 3) & ~3; }
+template <typename S>
+__host__ __device__ inline SeqLayout seq_layout_bwd(const KP<S>& p, int T) {
+  SeqLayout L;
+  const uint32_t V = sizeof(typename Fx<S>::Vec);
+  L.item = up128(p.gbB + p.nbB + (p.xs + p.us) * (uint32_t)sizeof(S));   // [B | Abar] | node block | xbar | ubar
+  L.vecA = up16(2 * up4(p.nu) * V);                               // (g; -ubar)
+  L.vecB = up16(up4(p.nx) * V);                                   // q
+  L.part = up16(T * (uint32_t)sizeof(typename Fx<S>::Acc));
+  return L;
+}
+template <typename S>
+__host__ __device__ inline SeqLayout seq_layout_fwd(const KP<S>& p, int T) {
+  SeqLayout L;
+  const uint32_t V = sizeof(typename Fx<S>::Vec);
+  L.item = up128(p.gfB + p.ktB + p.us * (uint32_t)sizeof(S));   // [Abar | B]^T | K^T of the parent | d of the node
+  L.vecA = up16(up4(p.nx + p.nu) * V);                   // (x; d) of the parent and of the node
+  L.vecB = L.vecA;
+  L.part = up16(T * (uint32_t)sizeof(typename Fx<S>::Acc));
+  return L;
+}
+
+// Barrier of the T working threads of a block.
+__device__ __forceinline__ void seq_bar(int T) { named_bar(1, T); }
+
+// Columns of a product: two blocks of n0 and n1, the second one from a warp
+// boundary on (both in one warp when they fit), so that no warp runs the sums
+// of both: with n0 = 50 and n1 = 20 packed into 70 threads, one warp ran 120
+// rows where the others ran 70.
+__host__ __device__ inline int seq_off(int n0, int n1) { return n0 + n1 <= 32 ? n0 : (n0 + 31) & ~31; }
+__host__ __device__ inline int seq_cols(int n0, int n1) { return (seq_off(n0, n1) + n1 + 31) & ~31; }
+
+// acc += sum over n rows of M[r] v[r]; `m` the shared-memory address of the
+// thread's entry in the first row, rows ldB bytes apart, `v` that of the
+// prepared vector (16-byte aligned).  Eight rows are loaded before their
+// products, without a branch among them.
+__device__ __forceinline__ void seq_rows(Fx<float>::Acc& acc, uint32_t m, uint32_t ldB, uint32_t v, int n) {
+  for (; n >= 8; n -= 8, m += 8 * ldB, v += 32) {
+    float a[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) a[i] = lds_f32(m + i * ldB);
+    const float4 x = lds_f32x4(v), y = lds_f32x4(v + 16);
+    acc.v = fmaf(a[0], x.x, acc.v);
+    acc.v = fmaf(a[1], x.y, acc.v);
+    acc.v = fmaf(a[2], x.z, acc.v);
+    acc.v = fmaf(a[3], x.w, acc.v);
+    acc.v = fmaf(a[4], y.x, acc.v);
+    acc.v = fmaf(a[5], y.y, acc.v);
+    acc.v = fmaf(a[6], y.z, acc.v);
+    acc.v = fmaf(a[7], y.w, acc.v);
+  }
+  if (n > 0) {
+    float a[7], x[7];
+#pragma unroll
+    for (int i = 0; i < 7; ++i) {
+      const int r = i < n ? i : n - 1;
+      a[i] = lds_f32(m + r * ldB);
+      x[i] = lds_f32(v + 4 * r);
+    }
+#pragma unroll
+    for (int i = 0; i < 7; ++i)
+      if (i < n) acc.v = fmaf(a[i], x[i], acc.v);
+  }
+}
+__device__ __forceinline__ void seq_rows(Fx<double>::Acc& acc, uint32_t m, uint32_t ldB, uint32_t v, int n) {
+  const char* mp = (const char*)__cvta_shared_to_generic(m);
+  const int4* vp = (const int4*)__cvta_shared_to_generic(v);
+  __builtin_assume(__isShared(mp));
+  __builtin_assume(__isShared(vp));
+#pragma unroll 4
+  for (int r = 0; r < n; ++r, mp += ldB) Fx<double>::mad(acc, *(const int2*)mp, vp[r]);
+}
+
+// Sum of the row groups' accumulators in the threads of row group 0 (one
+// barrier if there is more than one group; every thread calls it).
+template <typename S>
+__device__ __forceinline__ void seq_reduce(typename Fx<S>::Acc& acc, int rg, int RG, int CP, bool live,
+                                           typename Fx<S>::Acc* part, int T) {
+  if (RG == 1) return;
+  if (live && rg > 0) part[threadIdx.x] = acc;
+  seq_bar(T);
+  if (live && rg == 0)
+    for (int i = 1; i < RG; ++i) Fx<S>::add(acc, part[i * CP + threadIdx.x]);
+}
+
+// Largest key over threads 0 .. n - 1 (key is 0 elsewhere), to those threads;
+// a barrier when they span several warps.  FP32: nothing.
+template <typename S>
+__device__ __forceinline__ uint32_t seq_kmax(uint32_t key, int n, uint32_t* word, int T) {
+  if (sizeof(S) == 4) return 0u;
+  key = __reduce_max_sync(kFull, key);
+  if (n <= 32) return key;   // warp 0 holds all of them
+  const int w = threadIdx.x >> 5;
+  if ((threadIdx.x & 31) == 0 && w < 5) word[w] = key;
+  seq_bar(T);
+  const uint4 k4 = *reinterpret_cast<const uint4*>(word);
+  key = max(k4.x, k4.y);
+  if (n > 64) key = max(key, max(k4.z, k4.w));
+  if (n > 128) key = max(key, word[4]);
+  return key;
+}
+
+// The ring: per slot a barrier for "full" (the copies have arrived) and one for
+// "empty" (the T threads are through with it); a thread keeps the parity of its
+// next wait per slot.
+struct SeqRing {
+  uint64_t* full;
+  uint64_t* empty;
+  uint32_t phase;
+  bool dead;     // a wait gave up
+  __device__ __forceinline__ void wait(uint64_t* bar, int s, int32_t* err) {
+    if (dead) return;
+    if (mbar_wait(&bar[s], (phase >> s) & 1u)) {
+      phase ^= 1u << s;
+    } else {
+      dead = true;
+      atomicExch(err, 1);
+    }
+  }
+};
+
+// The fetching thread's loop: copies(slot, k, top) starts node k's copies
+// (top: the first node of a sequence); on return nothing is in flight
+// (bounded).
+template <typename F>
+__device__ __forceinline__ void seq_fetch(SeqRing& ring, const int32_t* stage_begin, int t_first, int t_last, int cnt,
+                                          int bid, int nblk, int D, int32_t* err, F copies) {
+  const int dt = t_first < t_last ? 1 : -1;
+  int slot = 0, issued = 0;
+  for (int ci = bid; ci < cnt && !ring.dead; ci += nblk) {
+    for (int t = t_first;; t += dt) {
+      const int k = stage_begin[t] + ci;
+      if (issued >= D) ring.wait(ring.empty, slot, err);
+      if (ring.dead) break;
+      fence_proxy_async();
+      copies(slot, k, t == t_first ? -1 : stage_begin[t - dt] + ci);
+      ++issued;
+      if (++slot == D) slot = 0;
+      if (t == t_last) break;
+    }
+  }
+  for (int s = 0; s < D; ++s) {
+    const int uses = (issued - s + D - 1) / D;
+    if (uses > 0) mbar_wait(&ring.full[s], (uint32_t)(uses - 1) & 1u);
+  }
+}
+
+// Sequences from stage t_hi down to t_lo, of which block bid of nblk takes
+// every nblk-th.
+template <typename S>
+__device__ __forceinline__ void bwd_seq_body(const KP<S>& p, int t_hi, int t_lo, int bid, int nblk, int D) {
+  if (p.skip && *p.skip) return;
+  using Mat = typename Fx<S>::Mat;
+  using Vec = typename Fx<S>::Vec;
+  using Acc = typename Fx<S>::Acc;
+  constexpr bool FX = sizeof(S) == 8;
+  constexpr uint32_t MB = sizeof(Mat), VB = sizeof(Vec);
+  extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ uint64_t bars[2][kMaxSlots];
+  __shared__ __align__(16) uint32_t kword[8];
+  __shared__ uint32_t kgs;
+  const int tid = threadIdx.x, T = blockDim.x - 32;
+  const int nx = p.nx, nu = p.nu, ncol = nx + nu;
+  const SeqLayout Ly = seq_layout_bwd(p, T);
+  const int cnt = p.stage_begin[t_lo + 1] - p.stage_begin[t_lo];
+  if (bid >= cnt) return;
+  SeqRing ring{bars[0], bars[1], 0u, false};
+  if (tid < 8) kword[tid] = 0;
+  if (tid == 0) {
+    for (int s = 0; s < D; ++s) {
+      mbar_init(&ring.full[s], 1);
+      mbar_init(&ring.empty[s], 1);
+    }
+    fence_mbar_init();
+  }
+  __syncthreads();
+  if (tid >= T) {
+    if (tid > T) return;
+    const uint32_t xB = p.xs * (uint32_t)sizeof(S), uB = p.us * (uint32_t)sizeof(S);
+    seq_fetch(ring, p.stage_begin, t_hi, t_lo, cnt, bid, nblk, D, p.err, [&](int slot, int k, int) {
+      const bool leaf = k >= p.nl;
+      unsigned char* dst = smem + slot * Ly.item;
+      uint64_t* bar = &ring.full[slot];
+      mbar_expect_tx(bar, xB + (leaf ? 0u : p.nbB + uB) + (k > 0 ? p.gbB : 0u));
+      if (!leaf) {
+        bulk_g2s(dst + p.gbB, p.pNB + (size_t)k * p.nbB, p.nbB, bar);
+        bulk_g2s(dst + p.gbB + p.nbB + xB, p.ubar + (size_t)k * p.us, uB, bar);
+      }
+      bulk_g2s(dst + p.gbB + p.nbB, p.xbar + (size_t)k * p.xs, xB, bar);
+      if (k > 0) bulk_g2s(dst, p.pGb + (size_t)(k - 1) * p.gbB, p.gbB, bar);
+    });
+    return;
+  }
+  Vec* const A = reinterpret_cast<Vec*>(smem + D * Ly.item);               // (g; -ubar), 4-entry aligned halves
+  Vec* const B = reinterpret_cast<Vec*>(smem + D * Ly.item + Ly.vecA);     // q
+  Acc* const part = reinterpret_cast<Acc*>(smem + D * Ly.item + Ly.vecA + Ly.vecB);
+  const uint32_t aA = smem_u32(A), aB = smem_u32(B), a0 = smem_u32(smem);
+  // column col of row group rg: d and h_u in columns 0 .. nu - 1, q and h_x from
+  // column off on; mc the column in the matrices [.. (nu) | .. (nx)]; row group
+  // rg takes rows u0 .. or x0 .. of a vector
+  const int off = seq_off(nu, nx), CP = seq_cols(nu, nx), RG = T / CP, rg = tid / CP, col = tid - rg * CP;
+  const bool inu = tid < nu, inx = tid >= off && tid < off + nx, own = inu || inx;
+  const bool live = rg < RG && (col < nu || (col >= off && col < off + nx));
+  const int mc = col < nu ? col : col - off + nu, ex = tid - off;
+  const int nu4 = up4(nu), cu = up4((nu + RG - 1) / RG), cx = up4((nx + RG - 1) / RG);
+  const int u0 = rg * cu, un = max(0, min(cu, nu - u0)), x0 = rg * cx, xn = max(0, min(cx, nx - x0));
+  S h = S(0);   // h of the current node: this thread's column
+  int slot = 0;
+  for (int ci = bid; ci < cnt; ci += nblk) {
+    for (int t = t_hi; t >= t_lo; --t) {
+      const int k = p.stage_begin[t] + ci;
+      const bool leaf = k >= p.nl;
+      if (t == t_hi && !leaf && own) {   // sum of the children's h, from the launch below
+        const int c0 = p.ch_begin[k], m = p.ch_count[k];
+        const S* src = p.hb + (int64_t)(c0 - 1) * p.hst + mc;
+        h = src[0];
+#pragma unroll 4
+        for (int c = 1; c < m; ++c) h += src[(int64_t)c * p.hst];
+      }
+      const unsigned char* it = smem + slot * Ly.item;
+      const uint32_t ait = a0 + slot * Ly.item;
+      const S* xb = reinterpret_cast<const S*>(it + p.gbB + p.nbB);
+      ring.wait(ring.full, slot, p.err);
+      S q = S(0);
+      if (leaf) {
+        if (inx) q = -xb[ex];
+      } else {
+        const S u = inu ? (xb + p.xs)[tid] : S(0);
+        const S g = inu ? u - h : S(0);
+        const S base = inx ? h - xb[ex] : S(0);
+        const uint32_t kg = seq_kmax<S>(inu ? max(Fx<S>::key(g), Fx<S>::key(u)) : 0u, nu, kword, T);
+        if (inu) {
+          A[tid] = Fx<S>::vec(g, kg);
+          A[nu4 + tid] = Fx<S>::vec(-u, kg);
+        }
+        if (FX && tid == 0) kgs = kg;
+        seq_bar(T);
+        Acc acc;
+        Fx<S>::zero(acc);
+        if (live) {   // [Rt^-1 | E] (nu x ncol), then K (nu x nx)
+          const uint32_t m1 = ait + p.gbB, m2 = m1 + nu * ncol * MB;
+          seq_rows(acc, m1 + (u0 * ncol + mc) * MB, ncol * MB, aA + u0 * VB, un);
+          if (col >= off) seq_rows(acc, m2 + (u0 * nx + mc - nu) * MB, nx * MB, aA + (nu4 + u0) * VB, un);
+        }
+        seq_reduce<S>(acc, rg, RG, CP, live, part, T);
+        if (own) {
+          const int* xn_ = reinterpret_cast<const int*>(it + p.gbB + (nu * ncol + nu * nx) * MB);
+          const S v = Fx<S>::value(acc, FX ? Fx<S>::vec_exp(kgs) + xn_[mc] : 0);
+          if (inu) p.d[(int64_t)k * p.us + tid] = v;
+          else q = base + v;
+        }
+      }
+      if (k > 0) {
+        const uint32_t kq = seq_kmax<S>(inx ? Fx<S>::key(q) : 0u, CP, kword, T);
+        if (inx) B[ex] = Fx<S>::vec(q, kq);
+        seq_bar(T);
+        Acc acc;
+        Fx<S>::zero(acc);
+        if (live) seq_rows(acc, ait + (x0 * ncol + mc) * MB, ncol * MB, aB + x0 * VB, xn);
+        seq_reduce<S>(acc, rg, RG, CP, live, part, T);
+        if (own) {
+          h = Fx<S>::value(acc, FX ? Fx<S>::vec_exp(kq) + reinterpret_cast<const int*>(it + nx * ncol * MB)[mc] : 0);
+          if (t == t_lo) p.hb[(int64_t)(k - 1) * p.hst + mc] = h;
+        }
+        seq_bar(T);   // every thread is through with the slot and the vectors
+        if (tid == 0) mbar_arrive(&ring.empty[slot]);
+      }
+      if (++slot == D) slot = 0;
+    }
+  }
+}
+
+// Sequences from stage t_lo >= 1 down to the leaves' side t_hi.
+template <typename S>
+__device__ __forceinline__ void fwd_seq_body(const KP<S>& p, int t_lo, int t_hi, S* __restrict__ zo, int bid,
+                                             int nblk, int D) {
+  if (p.skip && *p.skip) return;
+  using Mat = typename Fx<S>::Mat;
+  using Vec = typename Fx<S>::Vec;
+  using Acc = typename Fx<S>::Acc;
+  constexpr bool FX = sizeof(S) == 8;
+  constexpr uint32_t MB = sizeof(Mat), VB = sizeof(Vec);
+  extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ uint64_t bars[2][kMaxSlots];
+  __shared__ __align__(16) uint32_t kword[2][8];
+  const int tid = threadIdx.x, T = blockDim.x - 32;
+  const int nx = p.nx, nu = p.nu, ncol = nx + nu;
+  const SeqLayout Ly = seq_layout_fwd(p, T);
+  const int cnt = p.stage_begin[t_lo + 1] - p.stage_begin[t_lo];
+  if (bid >= cnt) return;
+  SeqRing ring{bars[0], bars[1], 0u, false};
+  if (tid < 16) kword[tid >> 3][tid & 7] = 0;
+  if (tid == 0) {
+    for (int s = 0; s < D; ++s) {
+      mbar_init(&ring.full[s], 1);
+      mbar_init(&ring.empty[s], 1);
+    }
+    fence_mbar_init();
+  }
+  __syncthreads();
+  if (tid >= T) {
+    if (tid > T) return;
+    const uint32_t uB = p.us * (uint32_t)sizeof(S);
+    seq_fetch(ring, p.stage_begin, t_lo, t_hi, cnt, bid, nblk, D, p.err, [&](int slot, int k, int above) {
+      const bool leaf = k >= p.nl;
+      const int par = above < 0 ? p.parent[k] : above;
+      const bool first = above >= 0 || k == 1 || p.parent[k - 1] != par;   // k is its parent's first child
+      unsigned char* dst = smem + slot * Ly.item;
+      uint64_t* bar = &ring.full[slot];
+      mbar_expect_tx(bar, p.gfB + (first ? p.ktB : 0u) + (leaf ? 0u : uB));
+      bulk_g2s(dst, p.pGf + (size_t)(k - 1) * p.gfB, p.gfB, bar);
+      if (first) bulk_g2s(dst + p.gfB, p.pKt + (size_t)par * p.ktB, p.ktB, bar);
+      if (!leaf) bulk_g2s(dst + p.gfB + p.ktB, p.d + (size_t)k * p.us, uB, bar);
+    });
+    return;
+  }
+  Vec* W = reinterpret_cast<Vec*>(smem + D * Ly.item);              // (x; d) of the parent
+  Vec* Y = reinterpret_cast<Vec*>(smem + D * Ly.item + Ly.vecA);    // (x; d) of the node
+  Acc* const part = reinterpret_cast<Acc*>(smem + D * Ly.item + Ly.vecA + Ly.vecB);
+  const uint32_t a0 = smem_u32(smem);
+  // columns 0 .. nx - 1: x, from column off on: u of the parent; the threads of
+  // row group 0 also hold the entries of (x; d), entry e
+  const int off = seq_off(nx, nu), CP = seq_cols(nx, nu), RG = T / CP, rg = tid / CP, col = tid - rg * CP;
+  const bool inx = tid < nx, inu = tid >= off && tid < off + nu, own = inx || inu;
+  const int a = tid - off, e = inx ? tid : nx + a, ca = col - off;
+  const int cc = up4((ncol + RG - 1) / RG), cx = up4((nx + RG - 1) / RG);
+  const int w0 = rg * cc, wn = max(0, min(cc, ncol - w0)), x0 = rg * cx, xn = max(0, min(cx, nx - x0));
+  S w = S(0);   // entry tid of the parent's (x; d)
+  int ew = 0;   // exponent of W
+  int slot = 0;
+  for (int ci = bid; ci < cnt; ci += nblk) {
+    for (int t = t_lo; t <= t_hi; ++t) {
+      const int k = p.stage_begin[t] + ci;
+      const int par = t == t_lo ? p.parent[k] : p.stage_begin[t - 1] + ci;
+      const bool first = t > t_lo || k == 1 || p.parent[k - 1] != par;
+      const int64_t zxk = p.zx[k], zup = p.zu[par];
+      if (t == t_lo) {   // (x; d) of the parent, from the launch above
+        if (own) {
+          if (inu) w = p.d[(int64_t)par * p.us + a];
+          else if (par > 0) w = zo[p.zx[par] + tid];
+          else w = p.x0[tid];
+          if (par == 0 && first && inx) zo[p.zx[0] + tid] = w;
+        }
+        const uint32_t kw = seq_kmax<S>(own ? Fx<S>::key(w) : 0u, CP, kword[0], T);
+        if (own) W[e] = Fx<S>::vec(w, kw);
+        ew = Fx<S>::vec_exp(kw);
+        seq_bar(T);
+      }
+      const unsigned char* it = smem + slot * Ly.item;
+      const uint32_t ait = a0 + slot * Ly.item, aW = smem_u32(W);
+      ring.wait(ring.full, slot, p.err);
+      const bool live = rg < RG && (col < nx || (first && ca >= 0 && ca < nu));
+      Acc acc;
+      Fx<S>::zero(acc);
+      if (live) {   // [Abar | B]^T (ncol x nx) and K^T (nx x nu)
+        if (col < nx) seq_rows(acc, ait + (w0 * nx + col) * MB, nx * MB, aW + w0 * VB, wn);
+        else seq_rows(acc, ait + p.gfB + (x0 * nu + ca) * MB, nu * MB, aW + x0 * VB, xn);
+      }
+      seq_reduce<S>(acc, rg, RG, CP, live, part, T);
+      if (own && live) {
+        const int* ex = reinterpret_cast<const int*>(inx ? it + ncol * nx * MB : it + p.gfB + nx * nu * MB);
+        const S v = Fx<S>::value(acc, FX ? ew + ex[inx ? tid : a] : 0);
+        if (inx) {
+          zo[zxk + tid] = v;
+          w = v;
+        } else {
+          zo[zup + a] = w + v;
+        }
+      }
+      if (t < t_hi) {   // the node's (x; d) for the next step
+        if (inu) w = reinterpret_cast<const S*>(it + p.gfB + p.ktB)[a];
+        const uint32_t ky = seq_kmax<S>(own ? Fx<S>::key(w) : 0u, CP, kword[1], T);
+        if (own) Y[e] = Fx<S>::vec(w, ky);
+        ew = Fx<S>::vec_exp(ky);
+        Vec* y = W;
+        W = Y;
+        Y = y;
+      }
+      seq_bar(T);   // every thread is through with the slot, (x; d) complete
+      if (tid == 0) mbar_arrive(&ring.empty[slot]);
+      if (++slot == D) slot = 0;
+    }
+  }
+}
+
+template <typename S>
+__global__ void __launch_bounds__(kMaxSeqThreads + 32, 1) k_bwd_seq(KP<S> p, int t_hi, int t_lo, int D) {
+  bwd_seq_body<S>(p, t_hi, t_lo, blockIdx.x, gridDim.x, D);
+}
+template <typename S>
+__global__ void __launch_bounds__(kMaxSeqThreads + 32, 1) k_fwd_seq(KP<S> p, int t_lo, int t_hi, S* __restrict__ zo,
+                                                            int D) {
+  fwd_seq_body<S>(p, t_lo, t_hi, zo, blockIdx.x, gridDim.x, D);
+}
+
+// Batched: block -> (instance, block) from the launch's map; stage < 0: the
+// chain region of every instance (forward: below the root at the earliest).
+template <typename S>
+__global__ void __launch_bounds__(kMaxSeqThreads + 32, 1) k_bwd_seq_b(const BInst<S>* __restrict__ bi, BMap m) {
+  const int i = m.inst[blockIdx.x], t = m.stage[i];
+  const KP<S> p = bi[i].kp;
+  bwd_seq_body<S>(p, t < 0 ? p.N : t, t < 0 ? p.chain_stage : t, blockIdx.x - m.base[i], m.cnt[i], 1);
+}
+template <typename S>
+__global__ void __launch_bounds__(kMaxSeqThreads + 32, 1) k_fwd_seq_b(const BInst<S>* __restrict__ bi, BMap m) {
+  const int i = m.inst[blockIdx.x], t = m.stage[i];
+  const KP<S> p = bi[i].kp;
+  const int top = p.chain_stage > 0 ? p.chain_stage : 1;
+  fwd_seq_body<S>(p, t < 0 ? top : t, t < 0 ? p.N : t, bi[i].TVt, blockIdx.x - m.base[i], m.cnt[i], 1);
+}
+
+// ---------------------------------------------------------------------------
+// launch shapes
+// ---------------------------------------------------------------------------
+static size_t max_dyn_smem() {
+  static size_t v = 0;
+  if (!v) {
+    int dev = 0, b = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&b, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    v = (size_t)b;
+  }
+  return v;
+}
+static int num_sms() {
+  static int v = 0;
+  if (!v) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+  }
+  return v;
+}
+
+// Threads per block (without the fetching warp): a multiple of 32 that covers
+// the widest product, times row groups that shorten the serial sums.  Two row
+// groups where few sequences leave most of an SM to a block and the sums are
+// long enough to pay for the barrier between them (FP64, nx >= 12: 3.5 against
+// 4.0 us a backward step at nx = 50, nu = 20; FP32 1.36 against 1.31 us); one
+// where many blocks share an SM (FP64, 62,805 nodes: 670 us a backward chain
+// pass against 1,029 us).
+static int seq_threads(int nx, int nu, bool f64, bool many) {
+  const int CP = std::max(seq_cols(nx, nu), seq_cols(nu, nx));
+  const int rg = f64 && !many && nx >= 12 ? 2 : 1;
+  return std::min(kMaxSeqThreads / CP, rg) * CP;
+}
+
+struct SeqShape {
+  int T, D, grid;
+  size_t bytes;
+};
+
+// Threads, slots and grid for `cnt` sequences of Lq nodes.  More than two
+// sequences per SM: one slot, and as many blocks as are resident -- at nx = 50,
+// nu = 20 four FP64 or eight FP32 ones, which hide one another's copies
+// better than a second slot does with half the blocks (FP64 chains of the
+// 62,805-node tree: 670 against 957 us).  Fewer: a second slot, if the
+// sequences are longer than one node and it fits.
+template <typename S, typename F>
+static SeqShape seq_shape(const KP<S>& p, int cnt, int Lq, F layout) {
+  SeqShape s;
+  const int sms = num_sms();
+  const bool many = cnt > 2 * sms;
+  s.T = seq_threads(p.nx, p.nu, sizeof(S) == 8, many);
+  const SeqLayout L = layout(p, s.T);
+  s.D = !many && Lq > 1 ? 2 : 1;
+  while (s.D > 1 && L.bytes(s.D) > max_dyn_smem() - 512) --s.D;
+  s.bytes = L.bytes(s.D);
+  const int by_smem = (int)(228 * 1024 / (s.bytes + 1280));   // static part and the 1 KB of the system
+  const int regs = sizeof(S) == 8 ? 112 : 80;
+  const int by_thr = std::min(2048 / (s.T + 32), 65536 / ((s.T + 32) * regs));
+  const int blocks = std::max(1, std::min(32, std::min(by_smem, by_thr)));
+  s.grid = std::max(1, std::min(cnt, sms * blocks));
+  return s;
+}
+
+// Raises a kernel's dynamic shared-memory limit, once per kernel and device.
+template <typename F>
+static void allow_smem(F* fn, std::atomic<uint64_t>& done) {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  const uint64_t bit = 1ull << (dev & 63);
+  if (done.load(std::memory_order_acquire) & bit) return;
+  cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(max_dyn_smem() - 512));
+  done.fetch_or(bit, std::memory_order_release);
+}
+
+template <typename S>
+int launch_bwd_seq(const KP<S>& p, int t_hi, int t_lo, int cnt, cudaStream_t st) {
+  const SeqShape s = seq_shape(p, cnt, t_hi - t_lo + 1, [](const KP<S>& q, int T) { return seq_layout_bwd(q, T); });
+  static std::atomic<uint64_t> done{0};
+  allow_smem(k_bwd_seq<S>, done);
+  k_bwd_seq<S><<<s.grid, s.T + 32, s.bytes, st>>>(p, t_hi, t_lo, s.D);
+  return 1;
+}
+template <typename S>
+int launch_fwd_seq(const KP<S>& p, int t_lo, int t_hi, int cnt, S* zo, cudaStream_t st) {
+  const SeqShape s = seq_shape(p, cnt, t_hi - t_lo + 1, [](const KP<S>& q, int T) { return seq_layout_fwd(q, T); });
+  static std::atomic<uint64_t> done{0};
+  allow_smem(k_fwd_seq<S>, done);
+  k_fwd_seq<S><<<s.grid, s.T + 32, s.bytes, st>>>(p, t_lo, t_hi, zo, s.D);
+  return 1;
+}
+
+// One shape for a batch: the most threads and shared memory over the
+// instances.  Returns false if some instance's layout does not fit.
+template <typename S>
+bool seq_batch_shape(const std::vector<KP<S>>& kps, SeqBatchShape& sh) {
+  sh.T = 32;
+  for (const KP<S>& p : kps) sh.T = std::max(sh.T, seq_threads(p.nx, p.nu, sizeof(S) == 8, true));
+  sh.bytes_bwd = sh.bytes_fwd = 0;
+  for (const KP<S>& p : kps) {
+    sh.bytes_bwd = std::max(sh.bytes_bwd, seq_layout_bwd(p, sh.T).bytes(1));
+    sh.bytes_fwd = std::max(sh.bytes_fwd, seq_layout_fwd(p, sh.T).bytes(1));
+  }
+  return std::max(sh.bytes_bwd, sh.bytes_fwd) <= max_dyn_smem() - 512;
+}
+
+// which = 0 backward chains, 1 backward stage, 2 forward stage, 3 forward chains
+template <typename S>
+void launch_seq_b(int which, const BInst<S>* bi, const BMap& m, int nblocks, const SeqBatchShape& sh,
+                  cudaStream_t st) {
+  if (nblocks <= 0) return;
+  if (which <= 1) {
+    static std::atomic<uint64_t> done{0};
+    allow_smem(k_bwd_seq_b<S>, done);
+    k_bwd_seq_b<S><<<nblocks, sh.T + 32, sh.bytes_bwd, st>>>(bi, m);
+  } else {
+    static std::atomic<uint64_t> done{0};
+    allow_smem(k_fwd_seq_b<S>, done);
+    k_fwd_seq_b<S><<<nblocks, sh.T + 32, sh.bytes_fwd, st>>>(bi, m);
+  }
+}
+
+#define SPOCK_SEQ_INST(S)                                                                            \
+  template int launch_bwd_seq<S>(const KP<S>&, int, int, int, cudaStream_t);                         \
+  template int launch_fwd_seq<S>(const KP<S>&, int, int, int, S*, cudaStream_t);                     \
+  template bool seq_batch_shape<S>(const std::vector<KP<S>>&, SeqBatchShape&);                       \
+  template void launch_seq_b<S>(int, const BInst<S>*, const BMap&, int, const SeqBatchShape&, cudaStream_t);
+SPOCK_SEQ_INST(double)
+SPOCK_SEQ_INST(float)
+
+}  // namespace spock

@@ -32,8 +32,8 @@ void launch_lstar(const KP<S>& p, const S* eta, S* zout, int grid, cudaStream_t 
 void launch_reduce_stats(const double* pd, int nd, const double* pp, int np, double* out, cudaStream_t st,
                          const int32_t* skip = nullptr);
 template <typename S>
-int launch_riccati(const KP<S>& p, const std::vector<int32_t>& stage_begin, const std::vector<int32_t>& stage_maxch,
-                   S* zo, cudaStream_t st, cudaEvent_t* ev);
+int launch_riccati(const KP<S>& p, const std::vector<int32_t>& stage_begin, S* zo, cudaStream_t st,
+                   cudaEvent_t* ev);
 
 enum { DM_APPLY_L_ = 0, DM_PROXG_ = 1, DM_DUAL_ = 2 };
 
@@ -297,6 +297,16 @@ static KP<S> make_kp(const Problem& P, double alpha, const int32_t* stage_begin_
   k.Gf = f.Gf;
   k.NB = f.NB;
   k.Kt = f.Kt;
+  k.pGb = f.pGb;
+  k.pGf = f.pGf;
+  k.pNB = f.pNB;
+  k.pKt = f.pKt;
+  k.gbB = f.gbB;
+  k.gfB = f.gfB;
+  k.nbB = f.nbB;
+  k.ktB = f.ktB;
+  k.hb = f.hb;
+  k.hst = f.hst;
   k.qs = f.qs;
   k.rs = f.rs;
   k.qns = f.qns;
@@ -416,7 +426,7 @@ static void eval_T(const Ctx& c, const S* v, S* Tv, const S* dir, double* stats,
   if (ev) record_event(ev[0], c.st);
   launch_prep<S>(kp, v, v + nz, Tv, maxb, c.st);
   if (ev) record_event(ev[1], c.st);
-  int launches = 2 + launch_riccati<S>(kp, P.tree.stage_begin, P.tree.stage_maxch, Tv, c.st, ev ? ev + 2 : nullptr);
+  int launches = 2 + launch_riccati<S>(kp, P.tree.stage_begin, Tv, c.st, ev ? ev + 2 : nullptr);
   if (ev) record_event(ev[5], c.st);
   launch_dual<S>(kp, DM_DUAL_, stats != nullptr, v, Tv, v + nz, Tv + nz, dir, ws ? ws->pd : nullptr,
                  ws ? ws->grid_d : std::min((P.tree.n + 3) / 4, maxb), c.st);
@@ -891,10 +901,10 @@ struct Batch {
   std::vector<void*> p_ws;
   std::vector<double> p_alpha;
   void* bi_dev = nullptr;  // BInst<S>[n]
-  DevMap node, vec, chain_b, chain_f;
+  DevMap node, vec, chains;
   std::vector<DevMap> bwd_lv, fwd_lv;  // branching stages, one map per level
   int fam = 0;                         // Riccati kernels: 0 direct, 1 staged (bulk copies)
-  TmaBatchShape tsh;
+  SeqBatchShape tsh;
   int J = 1, SL = 1;
   int launches_per_eval = 0;
   // graph of kBatchRounds rounds
@@ -985,7 +995,7 @@ static void batch_plan(Batch& B, const std::vector<Workspace*>& wss, const std::
   const int n = (int)B.probs.size();
   std::vector<BInst<S>> h(n);
   std::vector<int> cn(n), cv(n);
-  int max_cs = 0, max_ch = 1;
+  int max_cs = 0;
   B.J = 1;
   B.SL = 1;
   for (int i = 0; i < n; ++i) {
@@ -1000,7 +1010,6 @@ static void batch_plan(Batch& B, const std::vector<Workspace*>& wss, const std::
     cn[i] = b.nb_node;
     cv[i] = b.nb_vec;
     max_cs = std::max(max_cs, (int)P.tree.chain_stage);
-    for (int t = 0; t < P.tree.chain_stage; ++t) max_ch = std::max(max_ch, (int)P.tree.stage_maxch[t]);
     B.J = std::max(B.J, (P.nx + P.nu + 2 + 31) / 32);
     B.SL = std::max(B.SL, (P.nx + P.nu + 31) / 32);
   }
@@ -1010,22 +1019,20 @@ static void batch_plan(Batch& B, const std::vector<Workspace*>& wss, const std::
   if (B.fam == 1) {
     std::vector<KP<S>> kps(n);
     for (int i = 0; i < n; ++i) kps[i] = h[i].kp;
-    if (!tma_batch_shape<S>(kps, max_ch, B.tsh)) B.fam = 0;
+    if (!seq_batch_shape<S>(kps, B.tsh)) B.fam = 0;
   }
-  const int cw_b = B.fam == 1 ? B.tsh.wpb_bwd : kWarpsPerBlock;  // chains per chain block
-  const int cw_f = B.fam == 1 ? B.tsh.wpb_fwd : kWarpsPerBlock;
-  const int npb = B.fam == 1 ? 1 : kWarpsPerBlock;                // branching nodes per stage block
-  std::vector<int> ccb(n), ccf(n);
+  const int npb = B.fam == 1 ? 1 : kWarpsPerBlock;   // chains or branching nodes per block
+  std::vector<int> cc(n);
   for (int i = 0; i < n; ++i) {
     const KP<S>& k = h[i].kp;
-    const bool chains = k.n_chains > 0 && k.chain_stage < k.N;
-    ccb[i] = chains ? (k.n_chains + cw_b - 1) / cw_b : 0;
-    ccf[i] = chains ? (k.n_chains + cw_f - 1) / cw_f : 0;
+    const Tree& t = B.probs[i]->tree;
+    // the sequence kernels also take the leaves of a tree without chains
+    const bool chains = B.fam == 1 || (k.n_chains > 0 && k.chain_stage < k.N);
+    cc[i] = chains ? (t.stage_begin[t.chain_stage + 1] - t.stage_begin[t.chain_stage] + npb - 1) / npb : 0;
   }
   B.node = B.make_map(cn, {});
   B.vec = B.make_map(cv, {});
-  B.chain_b = B.make_map(ccb, {});
-  B.chain_f = B.make_map(ccf, {});
+  B.chains = B.make_map(cc, {});
   for (int L = 0; L < max_cs; ++L) {  // backward: level L is stage cs_i - 1 - L of instance i
     std::vector<int> cnt(n, 0), stg(n, -1);
     for (int i = 0; i < n; ++i) {
@@ -1042,7 +1049,7 @@ static void batch_plan(Batch& B, const std::vector<Workspace*>& wss, const std::
     std::vector<int> cnt(n, 0), stg(n, -1);
     for (int i = 0; i < n; ++i) {
       const Tree& t = B.probs[i]->tree;
-      if (L < t.chain_stage) {
+      if (L < t.chain_stage && !(B.fam == 1 && L == 0)) {   // the staged forward pass starts at stage 1
         stg[i] = L;
         cnt[i] = (t.stage_begin[L + 1] - t.stage_begin[L] + npb - 1) / npb;
       }
@@ -1065,15 +1072,15 @@ static void batch_eval(Batch& B, cudaStream_t st) {
   const BInst<S>* bi = (const BInst<S>*)B.bi_dev;
   launch_node_ops_b<S>(0, bi, B.node.view(n), B.node.nblocks, n, B.J, st);
   if (B.fam == 1) {
-    launch_riccati_tma_b<S>(0, bi, B.chain_b.view(n), B.chain_b.nblocks, B.SL, B.tsh, st);
-    for (const DevMap& m : B.bwd_lv) launch_riccati_tma_b<S>(1, bi, m.view(n), m.nblocks, B.SL, B.tsh, st);
-    for (const DevMap& m : B.fwd_lv) launch_riccati_tma_b<S>(2, bi, m.view(n), m.nblocks, B.SL, B.tsh, st);
-    launch_riccati_tma_b<S>(3, bi, B.chain_f.view(n), B.chain_f.nblocks, B.SL, B.tsh, st);
+    launch_seq_b<S>(0, bi, B.chains.view(n), B.chains.nblocks, B.tsh, st);
+    for (const DevMap& m : B.bwd_lv) launch_seq_b<S>(1, bi, m.view(n), m.nblocks, B.tsh, st);
+    for (const DevMap& m : B.fwd_lv) launch_seq_b<S>(2, bi, m.view(n), m.nblocks, B.tsh, st);
+    launch_seq_b<S>(3, bi, B.chains.view(n), B.chains.nblocks, B.tsh, st);
   } else {
-    launch_riccati_b<S>(0, bi, B.chain_b.view(n), B.chain_b.nblocks, B.SL, st);
+    launch_riccati_b<S>(0, bi, B.chains.view(n), B.chains.nblocks, B.SL, st);
     for (const DevMap& m : B.bwd_lv) launch_riccati_b<S>(1, bi, m.view(n), m.nblocks, B.SL, st);
     for (const DevMap& m : B.fwd_lv) launch_riccati_b<S>(2, bi, m.view(n), m.nblocks, B.SL, st);
-    launch_riccati_b<S>(3, bi, B.chain_f.view(n), B.chain_f.nblocks, B.SL, st);
+    launch_riccati_b<S>(3, bi, B.chains.view(n), B.chains.nblocks, B.SL, st);
   }
   launch_node_ops_b<S>(1, bi, B.node.view(n), B.node.nblocks, n, B.J, st);
   launch_node_ops_b<S>(3, bi, B.node.view(n), 0, n, B.J, st);
@@ -1606,7 +1613,7 @@ static int adjoint_impl(Problem& P, const double* z, const double* eta, const do
     launch_lstar<double>(kp, q, t, gnode, st);
     launch_axpy(nz, 2.0 * alpha, t, x, r, gvec, st);
     launch_prep<double>(kA, r, zero_eta, pv, maxb, st);
-    launch_riccati<double>(kA, P.tree.stage_begin, P.tree.stage_maxch, pv, st, nullptr);
+    launch_riccati<double>(kA, P.tree.stage_begin, pv, st, nullptr);
     launch_dual<double>(kp, DM_APPLY_L_, false, pv, nullptr, nullptr, Lp, nullptr, nullptr, gnode, st);
   };
   auto apply_op = [&](const double* x, double* out) {   // out = (I - J^T) x
@@ -1757,6 +1764,78 @@ static int32_t pad16(int64_t elems, size_t elt) {
   return (int32_t)((elems + a - 1) / a * a);
 }
 
+// One kind of factor block of the sequence kernels (KP in kernels.cuh), built
+// from the FP64 factors on the device: one thread per column of a block.
+enum BlockKind : int { BK_GB = 0, BK_NB = 1, BK_GF = 2, BK_KT = 3 };
+template <typename S>
+__global__ void k_factor_blocks(int kind, int nx, int nu, const double* __restrict__ in, int64_t stride,
+                                unsigned char* __restrict__ out, int64_t blockB, int64_t count) {
+  using Mat = typename Fx<S>::Mat;
+  const int ncol = nx + nu;
+  const int nrow = kind == BK_GB ? nx : (kind == BK_NB ? 2 * nu : (kind == BK_GF ? ncol : nx));
+  const int nc = kind == BK_GF ? nx : (kind == BK_KT ? nu : ncol);
+  const int64_t entries = kind == BK_NB ? (int64_t)nu * ncol + nu * nx : (int64_t)nrow * nc;
+  const int64_t total = count * nc;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t b = i / nc;
+    const int c = (int)(i % nc);
+    const double* a = in + b * stride;
+    Mat* o = reinterpret_cast<Mat*>(out + b * blockB);
+    auto entry = [&](int r) -> double {
+      if (kind == BK_GB) return a[(int64_t)r * ncol + (c < nu ? nx + c : c - nu)];
+      if (kind == BK_GF) return a[(int64_t)c * ncol + r];
+      if (kind == BK_KT) return a[(int64_t)c * nx + r];
+      const double* C = a + (int64_t)nu * nx;         // K + W^T
+      const double* Ri = C + (int64_t)nu * nx;
+      if (r >= nu) return c < nu ? 0.0 : a[(int64_t)(r - nu) * nx + (c - nu)];
+      if (c < nu) return Ri[(int64_t)r * nu + c];
+      double e = 0.0;
+      for (int q = 0; q < nu; ++q) e = fma(Ri[(int64_t)r * nu + q], C[(int64_t)q * nx + (c - nu)], e);
+      return e;
+    };
+    auto place = [&](int r) -> int64_t {
+      return kind == BK_NB && r >= nu ? (int64_t)nu * ncol + (int64_t)(r - nu) * nx + (c - nu) : (int64_t)r * nc + c;
+    };
+    const int nr = kind == BK_NB && c < nu ? nu : nrow;
+    if constexpr (sizeof(S) == 4) {
+      for (int r = 0; r < nr; ++r) o[place(r)] = (float)entry(r);
+    } else {
+      double big = 0.0;
+      for (int r = 0; r < nr; ++r) big = fmax(big, fabs(entry(r)));
+      // |entries| < 2^e; sums of more than 128 products get a bit of headroom
+      const int e = (big > 0.0 ? ilogb(big) + 1 : 0) + (nr > 128 ? 1 : 0);
+      reinterpret_cast<int32_t*>(o + entries)[c] = e;
+      for (int r = 0; r < nr; ++r) {
+        const long long v = llrint(scalbn(entry(r), 2 * kFxBits - e)), half = 1ll << (kFxBits - 1);
+        const int lo = (int)(((v + half) & ((1ll << kFxBits) - 1)) - half);
+        o[place(r)] = make_int2((int)((v - lo) >> kFxBits), lo);
+      }
+    }
+  }
+}
+
+// Builds the blocks of precision S (the FP64 factors are on the device).
+template <typename S>
+static void factor_blocks(Problem& P, DevFactors<S>& f) {
+  const DevFactors<double>& src = P.f64;
+  const int nx = P.nx, nu = P.nu, ncol = nx + nu;
+  const int64_t n1 = P.tree.n - 1, nl = P.tree.n_nonleaf;
+  auto build = [&](int kind, const double* in, int64_t stride, int64_t count, int64_t entries, int cols,
+                   uint32_t& blockB) {
+    blockB = up128((uint32_t)(entries * sizeof(typename Fx<S>::Mat) + (sizeof(S) == 8 ? cols * sizeof(int32_t) : 0)));
+    unsigned char* b = dalloc<unsigned char>(P, (size_t)count * blockB);
+    CUDA_TRY(cudaMemsetAsync(b, 0, (size_t)count * blockB));   // the padding is copied along
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((count * cols + 127) / 128, (int64_t)sm_count() * 16));
+    k_factor_blocks<S><<<grid, 128>>>(kind, nx, nu, in, stride, b, blockB, count);
+    check_launch();
+    return b;
+  };
+  f.pGb = build(BK_GB, src.Gb, src.gstride, n1, (int64_t)nx * ncol, ncol, f.gbB);
+  f.pGf = build(BK_GF, src.Gb, src.gstride, n1, (int64_t)nx * ncol, nx, f.gfB);
+  f.pNB = build(BK_NB, src.NB, src.nbstride, nl, (int64_t)nu * ncol + (int64_t)nu * nx, ncol, f.nbB);
+  f.pKt = build(BK_KT, src.NB, src.nbstride, nl, (int64_t)nx * nu, nu, f.ktB);
+}
+
 template <typename S>
 static void upload_factors(Problem& P, DevFactors<S>& f, const std::vector<double>& Gb,
                            const std::vector<double>& Gf, const std::vector<double>& NB,
@@ -1785,6 +1864,7 @@ static void upload_factors(Problem& P, DevFactors<S>& f, const std::vector<doubl
   f.Gf = upload(P, padded(Gf, (size_t)nx * ncol, f.gstride));
   f.NB = upload(P, padded(NB, 2 * (size_t)nu * nx + (size_t)nu * nu, f.nbstride));
   f.Kt = upload(P, padded(Kt, (size_t)nx * nu, f.ktstride));
+  factor_blocks<S>(P, f);
   f.qs = upload(P, cast(par[0]));
   f.rs = upload(P, cast(par[1]));
   f.qns = upload(P, cast(par[2]));
@@ -1826,6 +1906,8 @@ static void upload_factors(Problem& P, DevFactors<S>& f, const std::vector<doubl
   f.q = dalloc<S>(P, (size_t)t.n * f.xs);
   f.d = dalloc<S>(P, (size_t)t.n_nonleaf * f.us);
   f.x0 = dalloc<S>(P, (size_t)P.nx);
+  f.hst = pad16(ncol, sizeof(S));
+  f.hb = dalloc<S>(P, (size_t)(t.n - 1) * f.hst);
 }
 
 static bool all_finite(const double* a, size_t n) {
@@ -2473,7 +2555,7 @@ int spock_prox_f_dev(spock_problem* p, const double* x0_dev, double alpha, const
     KP<double> kp = op_kp(P, alpha);
     CUDA_TRY(cudaMemcpyAsync(P->f64.x0, x0_dev, sizeof(double) * P->nx, cudaMemcpyDeviceToDevice, st));
     launch_prep<double>(kp, z, (const double*)ws->zero_eta, z_out, sm_count() * 16, st);
-    launch_riccati<double>(kp, P->tree.stage_begin, P->tree.stage_maxch, z_out, st, nullptr);
+    launch_riccati<double>(kp, P->tree.stage_begin, z_out, st, nullptr);
     check_launch();
     CUDA_TRY(cudaStreamSynchronize(st));
     check_device_flag(*P, st);
@@ -2506,7 +2588,7 @@ int spock_T_dev(spock_problem* p, const double* x0_dev, double alpha, const doub
     KP<double> kp = op_kp(P, alpha);
     CUDA_TRY(cudaMemcpyAsync(P->f64.x0, x0_dev, sizeof(double) * P->nx, cudaMemcpyDeviceToDevice, st));
     launch_prep<double>(kp, z, eta, z_out, sm_count() * 16, st);
-    launch_riccati<double>(kp, P->tree.stage_begin, P->tree.stage_maxch, z_out, st, nullptr);
+    launch_riccati<double>(kp, P->tree.stage_begin, z_out, st, nullptr);
     launch_dual<double>(kp, DM_DUAL_, false, z, z_out, eta, eta_out, nullptr, nullptr,
                         std::min((P->tree.n + 3) / 4, sm_count() * 16), st);
     check_launch();
@@ -2718,6 +2800,7 @@ int spock_problem_clone(const spock_problem* base, spock_problem** out) {
         f.q = dalloc<S>(*C, (size_t)t.n * f.xs);
         f.d = dalloc<S>(*C, (size_t)t.n_nonleaf * f.us);
         f.x0 = dalloc<S>(*C, (size_t)C->nx);
+        f.hb = dalloc<S>(*C, (size_t)(t.n - 1) * f.hst);
       };
       scratch(C->f64, 0.0);
       scratch(C->f32, 0.0f);
@@ -2821,10 +2904,14 @@ extern "C" int spock_prox_f_noalloc_dev(spock_problem* p, const double* x0_dev, 
     kp.ubar = scratch + 2 * nxb;
     kp.d = scratch + 2 * nxb + nub;
     double* zero_eta = scratch + 2 * nxb + 2 * nub;
+    // the dual input is read by the preparation only; the Riccati passes then
+    // use its memory for the (n - 1) x hst numbers handed from node to parent
+    // (hst <= nx + nu + 2, the nonroot rows of eta)
+    kp.hb = zero_eta;
     // the array keeps the previous call's contents: the dual input must be zero
     CUDA_TRY(cudaMemsetAsync(zero_eta, 0, sizeof(double) * (size_t)P->off.n_eta, st));
     launch_prep<double>(kp, z, zero_eta, z_out, sm_count() * 16, st);
-    launch_riccati<double>(kp, P->tree.stage_begin, P->tree.stage_maxch, z_out, st, nullptr);
+    launch_riccati<double>(kp, P->tree.stage_begin, z_out, st, nullptr);
     check_launch();
     CUDA_TRY(cudaStreamSynchronize(st));
     check_device_flag(*P, st);

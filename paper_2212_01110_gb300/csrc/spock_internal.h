@@ -38,7 +38,6 @@ struct Tree {
   std::vector<int32_t> user_of, int_of;        // internal -> user, user -> internal
   std::vector<int32_t> parent, ch_begin, ch_count, stage, sib;  // internal
   std::vector<int32_t> stage_begin;            // [N + 2]
-  std::vector<int32_t> stage_maxch;            // [N + 1] most children of a node at each stage
   std::vector<double> prob;                    // internal, conditional
   // chain region: every node at stages >= chain_stage (and < N) has one child
   int32_t chain_stage = 0;
@@ -59,6 +58,9 @@ struct DevFactors {
   S* Gf = nullptr;   // [n-1][nx+nu][nx]  transpose of the above
   S* NB = nullptr;   // [nl][K (nu x nx) | K + W^T (nu x nx) | Rtilde^-1 (nu x nu)]
   S* Kt = nullptr;   // [nl][nx][nu]      K^T
+  // the factors in the blocks of the sequence kernels (KP in kernels.cuh)
+  unsigned char *pGb = nullptr, *pGf = nullptr, *pNB = nullptr, *pKt = nullptr;
+  uint32_t gbB = 0, gfB = 0, nbB = 0, ktB = 0;
   S* qs = nullptr;   // [n][nx]  sqrt(Q) of the edge into the node
   S* rs = nullptr;   // [n][nu]  sqrt(R)
   S* qns = nullptr;  // [n][nx]  sqrt(Q_N) (leaves)
@@ -88,6 +90,8 @@ struct DevFactors {
   S* q = nullptr;     // [n][nx]
   S* d = nullptr;     // [nl][nu]
   S* x0 = nullptr;    // [nx]
+  S* hb = nullptr;    // [n - 1][hst]
+  int32_t hst = 0;
   // per-node strides in elements, padded to a multiple of 16 bytes
   int32_t xs = 0, us = 0, gstride = 0, nbstride = 0, ktstride = 0;
 };
