@@ -45,8 +45,7 @@ struct BMap {
 };
 
 // ops.cu: which = 0 prox-f preparation (L* eta, proj_S2), 1 dual update with
-// the dual and primal statistics (warp per nonleaf node), 3 reduction of the
-// statistics (one block per instance; m unused).  J = lane slots for blocks
+// the dual and primal statistics (warp per nonleaf node).  J = lane slots for blocks
 // of nx + nu + 2.
 template <typename S>
 void launch_node_ops_b(int which, const BInst<S>* bi, const BMap& m, int nblocks, int n_inst, int J,
@@ -74,13 +73,11 @@ bool cta_supported(int nx, int nu, int mem);
 template <typename S>
 void launch_solve_cta(const BInst<S>* bi, int n_inst, int max_nxu, int mem, int64_t max_rounds, int32_t* trace,
                       cudaStream_t st);
-// rounds.cu: the four kernels of a round.
+// rounds.cu: the three kernels of a round.
 template <typename S>
 void launch_round_decide_b(const BInst<S>* bi, int n_inst, cudaStream_t st);
 template <typename S>
 void launch_round_commit_b(const BInst<S>* bi, const BMap& m, int nblocks, int mem, cudaStream_t st);
-template <typename S>
-void launch_round_aa_solve_b(const BInst<S>* bi, int n_inst, cudaStream_t st);
 template <typename S>
 void launch_round_point_b(const BInst<S>* bi, const BMap& m, int nblocks, int mem, cudaStream_t st);
 

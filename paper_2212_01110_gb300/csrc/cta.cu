@@ -41,7 +41,10 @@ __device__ __forceinline__ void cta_eval(const KP<S>& p, const BInst<S>& b) {
     fwd_chain_body<S, SL>(p, b.TVt, 0, 1);
     __syncthreads();
   }
-  dual_fused_body<S, true, J>(p, 0, 1, b.Vt, b.TVt, b.Vt + nz, b.TVt + nz, b.d, b.pd);
+  if (*reinterpret_cast<volatile int32_t*>(&b.st->pending) == P_LS)
+    dual_fused_body<S, true, J>(p, 0, 1, b.Vt, b.TVt, b.Vt + nz, b.TVt + nz, b.d, b.pd);
+  else
+    dual_fused_body<S, false, J>(p, 0, 1, b.Vt, b.TVt, b.Vt + nz, b.TVt + nz, b.d, b.pd);
   __syncthreads();
   reduce_stats_body(b.pd, 1, nullptr, 0, b.stats, p.skip);
   __syncthreads();

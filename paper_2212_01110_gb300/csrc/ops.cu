@@ -24,6 +24,7 @@
 #include "kernels.cuh"
 #include "ops_body.cuh"
 #include "spock_internal.h"
+#include "supermann.cuh"
 
 namespace spock {
 
@@ -45,8 +46,14 @@ template <typename S, bool DIR, int J>
 __global__ void __launch_bounds__(128, sizeof(S) == 4 ? 4 : 1)
     k_dual_fused(KP<S> p, const S* __restrict__ z, const S* __restrict__ zp,
                                                     const S* __restrict__ eta, S* __restrict__ out,
-                                                    const S* __restrict__ dir, double* __restrict__ partials) {
-  dual_fused_body<S, DIR, J>(p, blockIdx.x, gridDim.x, z, zp, eta, out, dir, partials);
+                                                    const S* __restrict__ dir, double* __restrict__ partials,
+                                                    const int32_t* pending) {
+  // the direction's inner products are read by the decision on a line-search
+  // trial only: other evaluations leave them out (and the reads of d)
+  if (DIR && pending && *pending != P_LS)
+    dual_fused_body<S, false, J>(p, blockIdx.x, gridDim.x, z, zp, eta, out, dir, partials);
+  else
+    dual_fused_body<S, DIR, J>(p, blockIdx.x, gridDim.x, z, zp, eta, out, dir, partials);
 }
 
 __global__ void k_reduce_stats(const double* __restrict__ pd, int nd, const double* __restrict__ pp, int np,
@@ -73,14 +80,12 @@ __global__ void __launch_bounds__(128) k_dual_b(const BInst<S>* __restrict__ bi,
   const int i = m.inst[blockIdx.x];
   const BInst<S>& b = bi[i];
   const KP<S> p = b.kp;
-  dual_fused_body<S, true, J>(p, blockIdx.x - m.base[i], m.cnt[i], b.Vt, b.TVt, b.Vt + p.n_z, b.TVt + p.n_z,
-                              b.d, b.pd);
-}
-
-template <typename S>
-__global__ void k_reduce_stats_b(const BInst<S>* __restrict__ bi) {
-  const BInst<S>& b = bi[blockIdx.x];
-  reduce_stats_body(b.pd, b.nb_node, nullptr, 0, b.stats, b.kp.skip);
+  if (b.st->pending == P_LS)
+    dual_fused_body<S, true, J>(p, blockIdx.x - m.base[i], m.cnt[i], b.Vt, b.TVt, b.Vt + p.n_z, b.TVt + p.n_z,
+                                b.d, b.pd);
+  else
+    dual_fused_body<S, false, J>(p, blockIdx.x - m.base[i], m.cnt[i], b.Vt, b.TVt, b.Vt + p.n_z, b.TVt + p.n_z,
+                                 b.d, b.pd);
 }
 
 // ---------------------------------------------------------------------------
@@ -134,7 +139,7 @@ void launch_prep(const KP<S>& p, const S* z, const S* eta, S* zo, int max_blocks
 
 template <typename S>
 void launch_dual(const KP<S>& p, int mode, bool stats, const S* z, const S* zp, const S* eta, S* out,
-                 const S* dir, double* partials, int grid, cudaStream_t st) {
+                 const S* dir, double* partials, int grid, cudaStream_t st, const int32_t* pending) {
   if (p.gen) {
     launch_dual_gen<S>(p, mode, stats, z, zp, eta, out, dir, partials, grid, st);
     return;
@@ -152,8 +157,8 @@ void launch_dual(const KP<S>& p, int mode, bool stats, const S* z, const S* zp, 
     switch (lane_slots(p.nx, p.nu)) {
 #define SPOCK_DF(JJ)                                                                                     \
   case JJ:                                                                                               \
-    if (dir) k_dual_fused<S, true, JJ><<<grid, 128, 0, st>>>(p, z, zp, eta, out, dir, partials);         \
-    else k_dual_fused<S, false, JJ><<<grid, 128, 0, st>>>(p, z, zp, eta, out, dir, partials);            \
+    if (dir) k_dual_fused<S, true, JJ><<<grid, 128, 0, st>>>(p, z, zp, eta, out, dir, partials, pending); \
+    else k_dual_fused<S, false, JJ><<<grid, 128, 0, st>>>(p, z, zp, eta, out, dir, partials, nullptr); \
     break;
       SPOCK_DF(1) SPOCK_DF(2) SPOCK_DF(3) SPOCK_DF(4)
       default: SPOCK_DF(kMaxJ)
@@ -180,10 +185,6 @@ void launch_reduce_stats(const double* pd, int nd, const double* pp, int np, dou
 template <typename S>
 void launch_node_ops_b(int which, const BInst<S>* bi, const BMap& m, int nblocks, int n_inst, int J,
                        cudaStream_t st) {
-  if (which == 3) {
-    k_reduce_stats_b<S><<<n_inst, 256, 0, st>>>(bi);
-    return;
-  }
 #define SPOCK_NB(JJ)                                                              \
   case JJ:                                                                        \
     if (which == 0) k_prep_b<S, JJ><<<nblocks, 128, 0, st>>>(bi, m);              \
@@ -201,9 +202,9 @@ template void launch_node_ops_b<float>(int, const BInst<float>*, const BMap&, in
 template void launch_prep<double>(const KP<double>&, const double*, const double*, double*, int, cudaStream_t);
 template void launch_prep<float>(const KP<float>&, const float*, const float*, float*, int, cudaStream_t);
 template void launch_dual<double>(const KP<double>&, int, bool, const double*, const double*, const double*,
-                                  double*, const double*, double*, int, cudaStream_t);
+                                  double*, const double*, double*, int, cudaStream_t, const int32_t*);
 template void launch_dual<float>(const KP<float>&, int, bool, const float*, const float*, const float*, float*,
-                                 const float*, double*, int, cudaStream_t);
+                                 const float*, double*, int, cudaStream_t, const int32_t*);
 template void launch_lstar<double>(const KP<double>&, const double*, double*, int, cudaStream_t);
 template void launch_lstar<float>(const KP<float>&, const float*, float*, int, cudaStream_t);
 

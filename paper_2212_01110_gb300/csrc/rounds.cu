@@ -2,11 +2,11 @@
 //
 // The buffers are fixed: (V, TV) the accepted iterate and T of it, (Vt, TVt)
 // the point being evaluated and T of it, d the direction, the Anderson columns.
-// Each round: k_round_decide reads the statistics of the last evaluation and
+// Each round: k_round_decide sums the statistics of the last evaluation and reads
 // the state, takes the SuperMann decision of Algorithm 3 (same readings as
 // supermann.cu) and writes this round's orders; k_round_commit copies an
 // accepted (Vt, TVt) into (V, TV) and in the
-// same pass writes the new Anderson column and its Gram row; k_round_aa_solve
+// same pass writes the new Anderson column and its Gram row; its last block
 // solves for gamma; k_round_point forms the next evaluation point in Vt
 // (v + d with the Anderson direction, v + tau d, the K2 point, or the relaxed
 // step); then T(Vt) is evaluated.  No decision is taken on the host, so a
@@ -15,14 +15,17 @@
 
 #include "batch.cuh"
 #include "kernels.cuh"
+#include "ops_body.cuh"
 #include "rounds_body.cuh"
 #include "supermann.cuh"
 
 namespace spock {
 
-__global__ void k_round_decide(SmState* st, const double* __restrict__ stats_t, int32_t* trace) {
-  if (threadIdx.x != 0) return;
-  round_decide_body(st, stats_t, trace);
+__global__ void __launch_bounds__(256) k_round_decide(SmState* st, const double* __restrict__ pd, int nd,
+                                                      double* stats_t, int32_t* trace) {
+  reduce_stats_body(pd, nd, nullptr, 0, stats_t, &st->done);
+  __syncthreads();
+  if (threadIdx.x == 0) round_decide_body(st, stats_t, trace);
 }
 
 template <typename S, int MEM>
@@ -31,11 +34,7 @@ __global__ void __launch_bounds__(256, 4) k_round_commit(SmState* st, S* __restr
                                                          S* __restrict__ MR, S* __restrict__ D, int64_t n,
                                                          int64_t ld, double* __restrict__ partials) {
   round_commit_body<S, MEM>(st, V, TV, Vt, TVt, MR, D, n, ld, partials, blockIdx.x, gridDim.x);
-}
-
-__global__ void __launch_bounds__(256) k_round_aa_solve(SmState* st, const double* __restrict__ partials,
-                                                        int nblocks) {
-  round_aa_solve_body(st, partials, nblocks);
+  if (MEM > 0) round_commit_last(st, partials, gridDim.x);
 }
 
 template <typename S, int MEM>
@@ -50,9 +49,11 @@ __global__ void __launch_bounds__(256) k_round_point(const SmState* __restrict__
 // batched rounds
 // ---------------------------------------------------------------------------
 template <typename S>
-__global__ void k_round_decide_b(const BInst<S>* __restrict__ bi, int n_inst) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n_inst) round_decide_body(bi[i].st, bi[i].stats, nullptr);
+__global__ void __launch_bounds__(256) k_round_decide_b(const BInst<S>* __restrict__ bi) {
+  const BInst<S>& b = bi[blockIdx.x];
+  reduce_stats_body(b.pd, b.nb_node, nullptr, 0, b.stats, b.kp.skip);
+  __syncthreads();
+  if (threadIdx.x == 0) round_decide_body(b.st, b.stats, nullptr);
 }
 template <typename S, int MEM>
 __global__ void __launch_bounds__(256, 4) k_round_commit_b(const BInst<S>* __restrict__ bi, BMap m) {
@@ -60,11 +61,7 @@ __global__ void __launch_bounds__(256, 4) k_round_commit_b(const BInst<S>* __res
   const BInst<S>& b = bi[i];
   round_commit_body<S, MEM>(b.st, b.V, b.TV, b.Vt, b.TVt, b.MR, b.D, b.n_v, b.ld, b.paa,
                             blockIdx.x - m.base[i], m.cnt[i]);
-}
-template <typename S>
-__global__ void __launch_bounds__(256) k_round_aa_solve_b(const BInst<S>* __restrict__ bi) {
-  const BInst<S>& b = bi[blockIdx.x];
-  round_aa_solve_body(b.st, b.paa, b.nb_vec);
+  if (MEM > 0) round_commit_last(b.st, b.paa, m.cnt[i]);
 }
 template <typename S, int MEM>
 __global__ void __launch_bounds__(256) k_round_point_b(const BInst<S>* __restrict__ bi, BMap m) {
@@ -74,11 +71,8 @@ __global__ void __launch_bounds__(256) k_round_point_b(const BInst<S>* __restric
                            m.cnt[i]);
 }
 
-void launch_round_decide(SmState* st, const double* stats_t, int32_t* trace, cudaStream_t s) {
-  k_round_decide<<<1, 32, 0, s>>>(st, stats_t, trace);
-}
-void launch_round_aa_solve(SmState* st, const double* partials, int nblocks, cudaStream_t s) {
-  k_round_aa_solve<<<1, 256, 0, s>>>(st, partials, nblocks);
+void launch_round_decide(SmState* st, const double* pd, int nd, double* stats_t, int32_t* trace, cudaStream_t s) {
+  k_round_decide<<<1, 256, 0, s>>>(st, pd, nd, stats_t, trace);
 }
 
 template <typename S>
@@ -107,11 +101,7 @@ void launch_round_point(SmState* st, const S* V, const S* TV, S* Vt, const S* TV
 
 template <typename S>
 void launch_round_decide_b(const BInst<S>* bi, int n_inst, cudaStream_t st) {
-  k_round_decide_b<S><<<(n_inst + 63) / 64, 64, 0, st>>>(bi, n_inst);
-}
-template <typename S>
-void launch_round_aa_solve_b(const BInst<S>* bi, int n_inst, cudaStream_t st) {
-  k_round_aa_solve_b<S><<<n_inst, 256, 0, st>>>(bi);
+  k_round_decide_b<S><<<n_inst, 256, 0, st>>>(bi);
 }
 template <typename S>
 void launch_round_commit_b(const BInst<S>* bi, const BMap& m, int nblocks, int mem, cudaStream_t st) {
@@ -135,7 +125,6 @@ void launch_round_point_b(const BInst<S>* bi, const BMap& m, int nblocks, int me
 }
 #define SPOCK_RB_INST(S)                                                                          \
   template void launch_round_decide_b<S>(const BInst<S>*, int, cudaStream_t);                     \
-  template void launch_round_aa_solve_b<S>(const BInst<S>*, int, cudaStream_t);                   \
   template void launch_round_commit_b<S>(const BInst<S>*, const BMap&, int, int, cudaStream_t);   \
   template void launch_round_point_b<S>(const BInst<S>*, const BMap&, int, int, cudaStream_t);
 SPOCK_RB_INST(double)

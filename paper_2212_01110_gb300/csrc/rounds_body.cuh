@@ -18,6 +18,13 @@ static __device__ void round_trace(SmState* st, int32_t* trace, int branch, int 
   }
 }
 
+// The next iteration; c2^k is kept as a running product (FP64 pow is some 100
+// instructions of 64 cycles each, in one thread that the GPU waits for).
+static __device__ __forceinline__ void round_next_k(SmState* st) {
+  st->k++;
+  st->c2k *= st->c2;
+}
+
 // Decisions after an iterate has been accepted (its statistics in stats_cur).
 static __device__ void round_after_accept(SmState* st, int32_t* trace) {
   const double* sc = st->stats_cur;
@@ -64,7 +71,7 @@ static __device__ void round_after_accept(SmState* st, int32_t* trace) {
     st->zeta = omega;
     round_trace(st, trace, 0, 0);
     st->n_k0++;
-    st->k++;
+    round_next_k(st);
     st->pending = P_K0;
     st->action = A_K0;
   } else {
@@ -75,7 +82,7 @@ static __device__ void round_after_accept(SmState* st, int32_t* trace) {
   }
 }
 
-static __device__ void round_decide_body(SmState* st, const double* __restrict__ stats_t, int32_t* trace) {
+static __device__ void round_decide_body(SmState* st, const double* stats_t, int32_t* trace) {
   st->op_accept = 0;
   st->op_aa = 0;
   st->op_point = PT_NONE;
@@ -96,10 +103,10 @@ static __device__ void round_decide_body(SmState* st, const double* __restrict__
       return;
     }
     if (omega <= st->omega_safe && omt <= st->c1 * omega) {  // K1
-      st->omega_safe = omt + pow(st->c2, (double)st->k);
+      st->omega_safe = omt + st->c2k;
       round_trace(st, trace, 1, st->nb);
       st->n_k1++;
-      st->k++;
+      round_next_k(st);
       accept = true;
     } else {
       const double rdM = stats_t[ST_RD] - st->alpha * (stats_t[ST_LRZ_DE] + stats_t[ST_RE_LDZ]);
@@ -109,7 +116,7 @@ static __device__ void round_decide_body(SmState* st, const double* __restrict__
         st->coef = st->lam * rho / (omt * omt);
         round_trace(st, trace, 2, st->nb);
         st->n_k2++;
-        st->k++;
+        round_next_k(st);
         st->op_point = PT_K2;
         st->pending = P_K2;
         st->action = A_K2;
@@ -120,7 +127,7 @@ static __device__ void round_decide_body(SmState* st, const double* __restrict__
         if (st->nb >= st->max_back) {  // cap: tau = 0, relaxed step v - lambda r
           round_trace(st, trace, 3, st->nb);
           st->n_cap++;
-          st->k++;
+          round_next_k(st);
           st->op_point = PT_KM;
           st->pending = P_K2;
           st->action = A_CAP;
@@ -236,98 +243,135 @@ __device__ __forceinline__ void round_commit_body(SmState* st, S* __restrict__ V
     }
   }
   if (MEM == 0 || !aa) return;
+  // row bid of the partials: [2 kMaxMemory], entries j < MEM of the Gram row and
+  // kMaxMemory + j of the right-hand side
   __shared__ double red[8][2 * kMaxMemory];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
-  for (int j = 0; j < MEM; ++j) {
-    const double a = warp_sum(gr[j]), b = warp_sum(rh[j]);
-    if (lane == 0) {
-      red[w][j] = a;
-      red[w][kMaxMemory + j] = b;
+  for (int g = 0; g < (2 * MEM + 7) / 8; ++g) {
+    double v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int e = 8 * g + i;
+      v[i] = e < MEM ? gr[e < MEM ? e : 0] : (e < 2 * MEM ? rh[e < 2 * MEM && e >= MEM ? e - MEM : 0] : 0.0);
     }
+    const double t = warp_sum8(v, lane);
+    const int e = 8 * g + warp_sum8_index(lane);
+    if ((lane & 3) == 0 && e < 2 * MEM) red[w][e < MEM ? e : kMaxMemory + e - MEM] = t;
   }
   __syncthreads();
-  if (threadIdx.x < 2 * kMaxMemory) {
-    const int j = threadIdx.x % kMaxMemory;
+  if (threadIdx.x < 2 * MEM) {
+    const int j = threadIdx.x < MEM ? threadIdx.x : kMaxMemory + threadIdx.x - MEM;
     double sum = 0.0;
-    if (j < cnt)
-      for (int ww = 0; ww < (int)(blockDim.x >> 5); ++ww) sum += red[ww][threadIdx.x];
-    partials[(int64_t)bid * 2 * kMaxMemory + threadIdx.x] = sum;
+    if ((j & (kMaxMemory - 1)) < cnt)
+      for (int ww = 0; ww < (int)(blockDim.x >> 5); ++ww) sum += red[ww][j];
+    partials[(int64_t)bid * 2 * kMaxMemory + j] = sum;
   }
 }
 
-
 // Gram update and least squares for gamma (FP64), newest columns first;
 // numerically singular Gram matrices drop their oldest columns from the solve.
+// One block.  A warp sums one value over the rows of the partials (lanes over
+// rows); then one warp factors L D L^T, lane a holding row a: one reciprocal
+// per pivot and products otherwise (a division or a square root is a chain of
+// some 10 FP64 instructions, 67 cycles each).
 __device__ __forceinline__ void round_aa_solve_body(SmState* st, const double* __restrict__ partials,
                                                     int nblocks) {
   if (!st->op_aa) return;
-  __shared__ double part[8][2 * kMaxMemory];
   __shared__ double sums[2 * kMaxMemory];
-  const int t = threadIdx.x;
-  const int ngrp = blockDim.x >> 5;  // 1..8 warps
-  {
-    const int val = t & 31, grp = t >> 5;
-    double s = 0.0;
-    for (int b = grp; b < nblocks; b += ngrp) s += partials[(int64_t)b * 2 * kMaxMemory + val];
-    part[grp][val] = s;
-  }
-  __syncthreads();
-  if (t < 2 * kMaxMemory) {
-    double s = 0.0;
-    for (int g = 0; g < ngrp; ++g) s += part[g][t];
-    sums[t] = s;
-  }
-  __syncthreads();
-  if (t != 0) return;
+  __shared__ double Mx[kMaxMemory][kMaxMemory + 1];   // row a: l_ab d_b for b < a, then the pivot d_a
+  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const int M = kMaxMemory, slot = st->aa_slot, cnt = st->aa_cnt, mem = st->mem;
-  for (int j = 0; j < cnt; ++j) {
-    st->G[slot * M + j] = sums[j];
-    st->G[j * M + slot] = sums[j];
-    st->rhs[j] = sums[M + j];
+  for (int v = threadIdx.x >> 5; v < 2 * cnt; v += nw) {
+    const int j = v < cnt ? v : M + v - cnt;
+    double s = 0.0;
+    for (int b = lane; b < nblocks; b += 32) s += __ldcg(partials + (int64_t)b * 2 * M + j);
+    s = warp_sum(s);
+    if (lane == 0) sums[j] = s;
   }
-  int order[kMaxMemory];
-  for (int j = 0; j < cnt; ++j) order[j] = ((slot - j) % mem + mem) % mem;
-  for (int j = 0; j < M; ++j) st->gamma[j] = 0.0;
-  st->aa_dropped = 0;
-  for (int use = cnt; use >= 1; --use) {
-    double Lm[kMaxMemory * kMaxMemory];
-    double maxd = 0.0;
-    for (int a = 0; a < use; ++a) maxd = fmax(maxd, st->G[order[a] * M + order[a]]);
-    bool ok = maxd > 0.0;
-    for (int a = 0; a < use && ok; ++a) {
-      for (int b = 0; b <= a; ++b) {
-        double s = st->G[order[a] * M + order[b]];
-        for (int c = 0; c < b; ++c) s -= Lm[a * M + c] * Lm[b * M + c];
-        if (a == b) {
-          if (!(s > 1e-13 * maxd)) {
-            ok = false;
-            break;
-          }
-          Lm[a * M + a] = sqrt(s);
-        } else {
-          Lm[a * M + b] = s / Lm[b * M + b];
-        }
+  __syncthreads();
+  if (threadIdx.x >= 32) return;
+  auto order = [&](int a) {   // a-th newest column
+    const int o = slot - a;
+    return o < 0 ? o + mem : o;
+  };
+  if (lane < cnt) {
+    st->G[slot * M + lane] = sums[lane];
+    st->G[lane * M + slot] = sums[lane];
+    st->rhs[lane] = sums[M + lane];
+  }
+  if (lane < M) st->gamma[lane] = 0.0;
+  __syncwarp();
+  const int oa = order(lane < cnt ? lane : 0);
+  double diag = lane < cnt ? st->G[oa * M + oa] : 0.0;
+  if (lane < cnt)
+    for (int b = 0; b <= lane; ++b) {
+      const int ob = order(b);
+      Mx[lane][b] = (oa == slot || ob == slot) ? sums[oa == slot ? ob : oa] : st->G[oa * M + ob];
+    }
+  if (lane < cnt && oa == slot) diag = sums[slot];
+  __syncwarp();
+  // factor while the pivots are positive: lane a's l_ab d_b - sum of products
+  int good = 0;   // pivots that could be formed
+  double inv = 0.0;
+  for (int c = 0; c < cnt; ++c) {
+    const double piv = Mx[c][c];
+    if (!(piv > 0.0)) break;
+    const double r = 1.0 / piv;
+    if (lane == c) inv = r;
+    if (lane > c && lane < cnt) {
+      const double l = Mx[lane][c] * r;
+      for (int b = c + 1; b <= lane; ++b) Mx[lane][b] = fma(-l, Mx[b][c], Mx[lane][b]);
+    }
+    __syncwarp();
+    good = c + 1;
+  }
+  // the most columns whose pivots are all above 1e-13 of their largest diagonal
+  int use = 0;
+  {
+    const double d = lane < good ? Mx[lane][lane] : 0.0;
+    double mx = diag;   // largest diagonal of the first lane + 1 columns
+    double mn = d;
+    for (int o = 1; o < 32; o <<= 1) {
+      const double up = __shfl_up_sync(kFull, mx, o), un = __shfl_up_sync(kFull, mn, o);
+      if (lane >= o) {
+        mx = fmax(mx, up);
+        mn = fmin(mn, un);
       }
     }
-    if (!ok) {
-      st->aa_dropped++;
-      continue;
-    }
-    double y[kMaxMemory];
-    for (int a = 0; a < use; ++a) {
-      double s = st->rhs[order[a]];
-      for (int c = 0; c < a; ++c) s -= Lm[a * M + c] * y[c];
-      y[a] = s / Lm[a * M + a];
-    }
-    for (int a = use - 1; a >= 0; --a) {
-      double s = y[a];
-      for (int c = a + 1; c < use; ++c) s -= Lm[c * M + a] * y[c];
-      y[a] = s / Lm[a * M + a];
-    }
-    for (int a = 0; a < use; ++a) st->gamma[order[a]] = y[a];
-    break;
+    const bool ok = lane < good && mn > 1e-13 * mx;
+    const unsigned okm = __ballot_sync(kFull, ok);
+    use = 32 - __clz(okm);
   }
+  if (lane == 0) st->aa_dropped = cnt - use;
+  if (use == 0) return;
+  // L y = rhs, then L^T gamma = D^-1 y
+  double y = lane < use ? sums[M + oa] : 0.0;
+  for (int c = 0; c < use; ++c) {
+    const double yc = __shfl_sync(kFull, y, c) * __shfl_sync(kFull, inv, c);
+    if (lane > c && lane < use) y = fma(-Mx[lane][c], yc, y);
+  }
+  y *= inv;
+  for (int c = use - 1; c > 0; --c) {
+    const double yc = __shfl_sync(kFull, y, c);
+    if (lane < c) y = fma(-Mx[c][lane] * inv, yc, y);
+  }
+  if (lane < use) st->gamma[oa] = y;
+}
+
+// After the commit: the block that finishes last solves for gamma (every
+// block of the grid calls it, all threads).
+__device__ __forceinline__ void round_commit_last(SmState* st, const double* __restrict__ partials, int nblk) {
+  if (!st->op_accept || !st->op_aa) return;
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(&st->ticket, 1u) == (unsigned)nblk - 1u;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  if (threadIdx.x == 0) st->ticket = 0;
+  round_aa_solve_body(st, partials, nblk);
 }
 
 

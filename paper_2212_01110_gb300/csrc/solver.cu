@@ -26,7 +26,7 @@ template <typename S>
 void launch_prep(const KP<S>& p, const S* z, const S* eta, S* zo, int max_blocks, cudaStream_t st);
 template <typename S>
 void launch_dual(const KP<S>& p, int mode, bool stats, const S* z, const S* zp, const S* eta, S* out,
-                 const S* dir, double* partials, int grid, cudaStream_t st);
+                 const S* dir, double* partials, int grid, cudaStream_t st, const int32_t* pending = nullptr);
 template <typename S>
 void launch_lstar(const KP<S>& p, const S* eta, S* zout, int grid, cudaStream_t st);
 void launch_reduce_stats(const double* pd, int nd, const double* pp, int np, double* out, cudaStream_t st,
@@ -236,7 +236,8 @@ static Workspace* get_ws_impl(Problem& P, int mem) {
     const int per_sm = (sizeof(S) == 8 && !P.general) ? 2 : 4;
     ws->grid_d = std::min((P.tree.n + kWarpsPerBlock - 1) / kWarpsPerBlock, sms * per_sm);
     ws->grid_d = std::max(ws->grid_d, 1);
-    ws->grid_v = sms * 4;
+    // the vector kernels of a round: four packs of 16 bytes a thread at least
+    ws->grid_v = (int)std::max<int64_t>(1, std::min<int64_t>(sms * 4, (ws->n_v * (int64_t)sizeof(S) + 16383) / 16384));
     ws->pd = (double*)ws->alloc(sizeof(double) * 8 * ws->grid_d);
     ws->paa = (double*)ws->alloc(sizeof(double) * 2 * kMaxMemory * ws->grid_v);
     ws->st = (SmState*)ws->alloc(sizeof(SmState));
@@ -415,7 +416,8 @@ struct Ctx {
 };
 
 template <typename S>
-static void eval_T(const Ctx& c, const S* v, S* Tv, const S* dir, double* stats, const int32_t* skip = nullptr) {
+static void eval_T(const Ctx& c, const S* v, S* Tv, const S* dir, double* stats, const int32_t* skip = nullptr,
+                   bool reduce = true, const int32_t* pending = nullptr) {
   Problem& P = *c.P;
   Workspace* ws = c.ws;
   KP<S> kp = make_kp<S>(P, c.alpha, c.stage_dev);
@@ -429,9 +431,9 @@ static void eval_T(const Ctx& c, const S* v, S* Tv, const S* dir, double* stats,
   int launches = 2 + launch_riccati<S>(kp, P.tree.stage_begin, Tv, c.st, ev ? ev + 2 : nullptr);
   if (ev) record_event(ev[5], c.st);
   launch_dual<S>(kp, DM_DUAL_, stats != nullptr, v, Tv, v + nz, Tv + nz, dir, ws ? ws->pd : nullptr,
-                 ws ? ws->grid_d : std::min((P.tree.n + 3) / 4, maxb), c.st);
+                 ws ? ws->grid_d : std::min((P.tree.n + 3) / 4, maxb), c.st, pending);
   if (ev) record_event(ev[6], c.st);
-  if (stats) {  // the dual kernel left the dual and primal statistics in pd
+  if (stats && reduce) {  // the dual kernel left the dual and primal statistics in pd
     launch_reduce_stats(ws->pd, ws->grid_d, nullptr, 0, stats, c.st, skip);
     launches += 1;
   }
@@ -707,6 +709,7 @@ static int solve_graph(Problem& P, const double* x0_dev, const spock_settings& s
   h.stall_window = stall_window;
   h.pending = P_INIT;
   h.n_T = 1;
+  h.c2k = 1.0;
   sm_init_state(ws->st, h, st);
   const int32_t* skip = &ws->st->done;
   // the graph of kRounds rounds (captured once per workspace and settings)
@@ -714,13 +717,12 @@ static int solve_graph(Problem& P, const double* x0_dev, const spock_settings& s
   auto round = [&](cudaStream_t s2) {
     Ctx c2 = c;
     c2.st = s2;
-    launch_round_decide(ws->st, stats_t, trace_dev, s2);
+    launch_round_decide(ws->st, ws->pd, ws->grid_d, stats_t, trace_dev, s2);   // sums the statistics as well
     launch_round_commit<S>(ws->st, V, TV, Vt, TVt, MR, Dm, nv, ws->ld, mem, ws->paa, grid_v, s2);
-    launch_round_aa_solve(ws->st, ws->paa, grid_v, s2);
     launch_round_point<S>(ws->st, V, TV, Vt, TVt, d, Dm, nv, ws->ld, mem, grid_v, s2);
     const int64_t before = ws->launches;
-    eval_T<S>(c2, Vt, TVt, d, stats_t, skip);
-    return 4 + (int)(ws->launches - before);
+    eval_T<S>(c2, Vt, TVt, d, stats_t, skip, false, &ws->st->pending);
+    return 3 + (int)(ws->launches - before);
   };
   ws->launches = 0;
   const int64_t max_rounds = (int64_t)(max_iter + 1) * (h.max_back + 3) + 2;
@@ -735,7 +737,7 @@ static int solve_graph(Problem& P, const double* x0_dev, const spock_settings& s
     ws->launches = 1;
   } else {
     CUDA_TRY(cudaEventRecord(ws->e0, st));
-    eval_T<S>(c, Vt, TVt, nullptr, stats_t, nullptr);  // T(v0); also sets kernel attributes outside capture
+    eval_T<S>(c, Vt, TVt, nullptr, stats_t, nullptr, false);  // T(v0); also sets kernel attributes outside capture
     const int64_t launches0 = ws->launches;
     const char* fam = getenv("SPOCK_RICCATI_KERNELS");
     const int trace_key = (trace_dev ? 1 : 0) + 2 * (s.profile ? 1 : 0) +
@@ -1056,7 +1058,7 @@ static void batch_plan(Batch& B, const std::vector<Workspace*>& wss, const std::
     }
     B.fwd_lv.push_back(B.make_map(cnt, stg));
   }
-  B.launches_per_eval = 5 + 2 * max_cs;
+  B.launches_per_eval = 4 + 2 * max_cs;
   B.p_prec = (int)sizeof(S);
   B.p_mem = mem;
   B.p_tile = tile;
@@ -1083,7 +1085,6 @@ static void batch_eval(Batch& B, cudaStream_t st) {
     launch_riccati_b<S>(3, bi, B.chains.view(n), B.chains.nblocks, B.SL, st);
   }
   launch_node_ops_b<S>(1, bi, B.node.view(n), B.node.nblocks, n, B.J, st);
-  launch_node_ops_b<S>(3, bi, B.node.view(n), 0, n, B.J, st);
   check_launch();
 }
 
@@ -1223,6 +1224,7 @@ static void batch_init(Batch& B, const std::vector<Workspace*>& wss, const std::
     h.mem = mem;
     h.pending = P_INIT;
     h.n_T = 1;
+    h.c2k = 1.0;
   }
   batch_states(B, wss, hs.data(), true, st);
 }
@@ -1249,7 +1251,6 @@ static void batch_rounds_direct(Batch& B, int mem, int rounds) {
   for (int r = 0; r < rounds; ++r) {
     launch_round_decide_b<S>(bi, n, B.main);
     launch_round_commit_b<S>(bi, B.vec.view(n), B.vec.nblocks, mem, B.main);
-    launch_round_aa_solve_b<S>(bi, n, B.main);
     launch_round_point_b<S>(bi, B.vec.view(n), B.vec.nblocks, mem, B.main);
     batch_eval<S>(B, B.main);
   }
@@ -1366,8 +1367,7 @@ static int batch_solve(Batch& B, const double* const* x0, const spock_settings& 
     for (int r = 0; r < kBatchRounds; ++r) {
       launch_round_decide_b<S>(bi, n, B.main);
       launch_round_commit_b<S>(bi, B.vec.view(n), B.vec.nblocks, mem, B.main);
-      launch_round_aa_solve_b<S>(bi, n, B.main);
-      launch_round_point_b<S>(bi, B.vec.view(n), B.vec.nblocks, mem, B.main);
+        launch_round_point_b<S>(bi, B.vec.view(n), B.vec.nblocks, mem, B.main);
       batch_eval<S>(B, B.main);
     }
     k_gather_done<<<(n + 127) / 128, 128, 0, B.main>>>(B.st_ptrs, n, B.done_dev);
@@ -1377,7 +1377,7 @@ static int batch_solve(Batch& B, const double* const* x0, const spock_settings& 
     cudaGraphDestroy(g);
     CUDA_TRY(e);
     B.g_alpha = a_key;
-    B.g_launches = kBatchRounds * (4 + B.launches_per_eval) + 1;
+    B.g_launches = kBatchRounds * (3 + B.launches_per_eval) + 1;
   }
   {
     std::vector<SmState*> h(n);

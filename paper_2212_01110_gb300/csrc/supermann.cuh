@@ -35,7 +35,9 @@ struct SmState {
   // what this round does, and whether the solve has finished
   int32_t pending, op_accept, op_aa, op_point;
   int32_t done, have_prev, aa_cnt, aa_next;
-  int32_t aa_slot, n_T, rounds, pad2_;
+  int32_t aa_slot, n_T, rounds;
+  uint32_t ticket;      // blocks of the commit kernel that have finished
+  double c2k;           // c2^k
   double stats_cur[8];
 };
 
@@ -43,15 +45,15 @@ struct SmState {
 enum SmPending : int32_t { P_INIT = 0, P_K0 = 1, P_LS = 2, P_K2 = 3 };
 enum SmPoint : int32_t { PT_NONE = 0, PT_DIR = 1, PT_LS = 2, PT_K2 = 3, PT_KM = 4 };
 
-// One round = decide (from the statistics of the last T evaluation) ->
-// commit/Anderson update -> Gram solve -> next evaluation point; the T
-// evaluation of that point follows (skipped once done).  Every kernel reads
-// its orders from the state, so the sequence can be captured in a graph.
-void launch_round_decide(SmState* st, const double* stats_t, int32_t* trace, cudaStream_t s);
+// One round = decide (from the statistics of the last T evaluation, whose
+// per-block rows pd [nd][8] it sums first) -> commit/Anderson update, its last
+// block solving for gamma -> next evaluation point; the T evaluation of that
+// point follows (skipped once done).  Every kernel reads its orders from the
+// state, so the sequence can be captured in a graph.
+void launch_round_decide(SmState* st, const double* pd, int nd, double* stats_t, int32_t* trace, cudaStream_t s);
 template <typename S>
 void launch_round_commit(SmState* st, S* V, S* TV, const S* Vt, const S* TVt, S* MR, S* D,
                          int64_t n, int64_t ld, int mem, double* partials, int grid, cudaStream_t s);
-void launch_round_aa_solve(SmState* st, const double* partials, int nblocks, cudaStream_t s);
 template <typename S>
 void launch_round_point(SmState* st, const S* V, const S* TV, S* Vt, const S* TVt, S* d, const S* D, int64_t n,
                         int64_t ld, int mem, int grid, cudaStream_t s);
