@@ -22,6 +22,7 @@
 // warp barriers inside the node loop.
 #include "batch.cuh"
 #include "kernels.cuh"
+#include "launch.cuh"
 #include "ops_body.cuh"
 #include "spock_internal.h"
 #include "supermann.cuh"
@@ -31,12 +32,14 @@ namespace spock {
 template <typename S, int MODE, int J>
 __global__ void __launch_bounds__(128) k_lstar(KP<S> p, const S* __restrict__ eta, const S* __restrict__ z,
                                                S* __restrict__ zo) {
+  pdl_enter();
   lstar_body<S, MODE, J>(p, blockIdx.x, gridDim.x, eta, z, zo);
 }
 
 template <typename S, int MODE, int J>
 __global__ void __launch_bounds__(128) k_dual(KP<S> p, const S* __restrict__ z, const S* __restrict__ zp,
                                               const S* __restrict__ eta, S* __restrict__ out) {
+  pdl_enter();
   dual_body<S, MODE, J>(p, blockIdx.x, gridDim.x, z, zp, eta, out);
 }
 
@@ -48,6 +51,7 @@ __global__ void __launch_bounds__(128, sizeof(S) == 4 ? 4 : 1)
                                                     const S* __restrict__ eta, S* __restrict__ out,
                                                     const S* __restrict__ dir, double* __restrict__ partials,
                                                     const int32_t* pending) {
+  pdl_enter();
   // the direction's inner products are read by the decision on a line-search
   // trial only: other evaluations leave them out (and the reads of d)
   if (DIR && pending && *pending != P_LS)
@@ -58,6 +62,7 @@ __global__ void __launch_bounds__(128, sizeof(S) == 4 ? 4 : 1)
 
 __global__ void k_reduce_stats(const double* __restrict__ pd, int nd, const double* __restrict__ pp, int np,
                                double* __restrict__ out, const int32_t* __restrict__ skip) {
+  pdl_enter();
   reduce_stats_body(pd, nd, pp, np, out, skip);
 }
 
@@ -69,6 +74,7 @@ __global__ void k_reduce_stats(const double* __restrict__ pd, int nd, const doub
 // ---------------------------------------------------------------------------
 template <typename S, int J>
 __global__ void __launch_bounds__(128) k_prep_b(const BInst<S>* __restrict__ bi, BMap m) {
+  pdl_enter();
   const int i = m.inst[blockIdx.x];
   const BInst<S>& b = bi[i];
   const KP<S> p = b.kp;
@@ -77,6 +83,7 @@ __global__ void __launch_bounds__(128) k_prep_b(const BInst<S>* __restrict__ bi,
 
 template <typename S, int J>
 __global__ void __launch_bounds__(128) k_dual_b(const BInst<S>* __restrict__ bi, BMap m) {
+  pdl_enter();
   const int i = m.inst[blockIdx.x];
   const BInst<S>& b = bi[i];
   const KP<S> p = b.kp;
@@ -102,22 +109,22 @@ inline int lane_slots(int nx, int nu) { return (nx + nu + 2 + 31) / 32; }
 template <typename S, int MODE>
 static void lstar_j(const KP<S>& p, const S* eta, const S* z, S* zo, int grid, cudaStream_t st) {
   switch (lane_slots(p.nx, p.nu)) {
-    case 1: k_lstar<S, MODE, 1><<<grid, 128, 0, st>>>(p, eta, z, zo); break;
-    case 2: k_lstar<S, MODE, 2><<<grid, 128, 0, st>>>(p, eta, z, zo); break;
-    case 3: k_lstar<S, MODE, 3><<<grid, 128, 0, st>>>(p, eta, z, zo); break;
-    case 4: k_lstar<S, MODE, 4><<<grid, 128, 0, st>>>(p, eta, z, zo); break;
-    default: k_lstar<S, MODE, kMaxJ><<<grid, 128, 0, st>>>(p, eta, z, zo); break;
+    case 1: launch_pdl(k_lstar<S, MODE, 1>, grid, 128, 0, st, p, eta, z, zo); break;
+    case 2: launch_pdl(k_lstar<S, MODE, 2>, grid, 128, 0, st, p, eta, z, zo); break;
+    case 3: launch_pdl(k_lstar<S, MODE, 3>, grid, 128, 0, st, p, eta, z, zo); break;
+    case 4: launch_pdl(k_lstar<S, MODE, 4>, grid, 128, 0, st, p, eta, z, zo); break;
+    default: launch_pdl(k_lstar<S, MODE, kMaxJ>, grid, 128, 0, st, p, eta, z, zo); break;
   }
 }
 
 template <typename S, int MODE>
 static void dual_j(const KP<S>& p, const S* z, const S* zp, const S* eta, S* out, int grid, cudaStream_t st) {
   switch (lane_slots(p.nx, p.nu)) {
-    case 1: k_dual<S, MODE, 1><<<grid, 128, 0, st>>>(p, z, zp, eta, out); break;
-    case 2: k_dual<S, MODE, 2><<<grid, 128, 0, st>>>(p, z, zp, eta, out); break;
-    case 3: k_dual<S, MODE, 3><<<grid, 128, 0, st>>>(p, z, zp, eta, out); break;
-    case 4: k_dual<S, MODE, 4><<<grid, 128, 0, st>>>(p, z, zp, eta, out); break;
-    default: k_dual<S, MODE, kMaxJ><<<grid, 128, 0, st>>>(p, z, zp, eta, out); break;
+    case 1: launch_pdl(k_dual<S, MODE, 1>, grid, 128, 0, st, p, z, zp, eta, out); break;
+    case 2: launch_pdl(k_dual<S, MODE, 2>, grid, 128, 0, st, p, z, zp, eta, out); break;
+    case 3: launch_pdl(k_dual<S, MODE, 3>, grid, 128, 0, st, p, z, zp, eta, out); break;
+    case 4: launch_pdl(k_dual<S, MODE, 4>, grid, 128, 0, st, p, z, zp, eta, out); break;
+    default: launch_pdl(k_dual<S, MODE, kMaxJ>, grid, 128, 0, st, p, z, zp, eta, out); break;
   }
 }
 
@@ -146,9 +153,9 @@ void launch_dual(const KP<S>& p, int mode, bool stats, const S* z, const S* zp, 
   }
   // operator-level modes (not on the solve path) use the widest lane layout
   if (mode == DM_APPLY_L) {
-    k_dual<S, DM_APPLY_L, kMaxJ><<<grid, 128, 0, st>>>(p, z, zp, eta, out);
+    launch_pdl(k_dual<S, DM_APPLY_L, kMaxJ>, grid, 128, 0, st, p, z, zp, eta, out);
   } else if (mode == DM_PROXG) {
-    k_dual<S, DM_PROXG, kMaxJ><<<grid, 128, 0, st>>>(p, z, zp, eta, out);
+    launch_pdl(k_dual<S, DM_PROXG, kMaxJ>, grid, 128, 0, st, p, z, zp, eta, out);
   } else if (!stats) {
     dual_j<S, DM_DUAL>(p, z, zp, eta, out, grid, st);
   } else {
@@ -157,8 +164,8 @@ void launch_dual(const KP<S>& p, int mode, bool stats, const S* z, const S* zp, 
     switch (lane_slots(p.nx, p.nu)) {
 #define SPOCK_DF(JJ)                                                                                     \
   case JJ:                                                                                               \
-    if (dir) k_dual_fused<S, true, JJ><<<grid, 128, 0, st>>>(p, z, zp, eta, out, dir, partials, pending); \
-    else k_dual_fused<S, false, JJ><<<grid, 128, 0, st>>>(p, z, zp, eta, out, dir, partials, nullptr); \
+    if (dir) launch_pdl(k_dual_fused<S, true, JJ>, grid, 128, 0, st, p, z, zp, eta, out, dir, partials, pending); \
+    else launch_pdl(k_dual_fused<S, false, JJ>, grid, 128, 0, st, p, z, zp, eta, out, dir, partials, nullptr); \
     break;
       SPOCK_DF(1) SPOCK_DF(2) SPOCK_DF(3) SPOCK_DF(4)
       default: SPOCK_DF(kMaxJ)
@@ -174,12 +181,12 @@ void launch_lstar(const KP<S>& p, const S* eta, S* zout, int grid, cudaStream_t 
     launch_lstar_gen<S>(p, LS_APPLY, eta, nullptr, zout, grid, st);
     return;
   }
-  k_lstar<S, LS_APPLY, kMaxJ><<<grid, 128, 0, st>>>(p, eta, nullptr, zout);
+  launch_pdl(k_lstar<S, LS_APPLY, kMaxJ>, grid, 128, 0, st, p, eta, nullptr, zout);
 }
 
 void launch_reduce_stats(const double* pd, int nd, const double* pp, int np, double* out, cudaStream_t st,
                          const int32_t* skip) {
-  k_reduce_stats<<<1, 256, 0, st>>>(pd, nd, pp, np, out, skip);
+  launch_pdl(k_reduce_stats, 1, 256, 0, st, pd, nd, pp, np, out, skip);
 }
 
 template <typename S>
@@ -187,8 +194,8 @@ void launch_node_ops_b(int which, const BInst<S>* bi, const BMap& m, int nblocks
                        cudaStream_t st) {
 #define SPOCK_NB(JJ)                                                              \
   case JJ:                                                                        \
-    if (which == 0) k_prep_b<S, JJ><<<nblocks, 128, 0, st>>>(bi, m);              \
-    else k_dual_b<S, JJ><<<nblocks, 128, 0, st>>>(bi, m);                         \
+    if (which == 0) launch_pdl(k_prep_b<S, JJ>, nblocks, 128, 0, st, bi, m);              \
+    else launch_pdl(k_dual_b<S, JJ>, nblocks, 128, 0, st, bi, m);                         \
     break;
   switch (J) {
     SPOCK_NB(1) SPOCK_NB(2) SPOCK_NB(3) SPOCK_NB(4)

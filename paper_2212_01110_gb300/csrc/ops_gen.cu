@@ -22,6 +22,7 @@
 // The cone projections of the cost epigraphs and the statistics are as in
 // the box form.
 #include "kernels.cuh"
+#include "launch.cuh"
 #include "ops_body.cuh"
 #include "spock_internal.h"
 
@@ -101,6 +102,7 @@ struct GenMats {
 template <typename S, int MODE, int J>
 __global__ void __launch_bounds__(128) k_lstar_g(KP<S> p, const S* __restrict__ eta, const S* __restrict__ z,
                                                  S* __restrict__ zo) {
+  pdl_enter();
   if (p.skip && *p.skip) return;
   const GenMats<S> G{p};
   const int lane = threadIdx.x & 31;
@@ -266,6 +268,7 @@ __global__ void __launch_bounds__(128) k_lstar_g(KP<S> p, const S* __restrict__ 
 template <typename S, int MODE, int J>
 __global__ void __launch_bounds__(128) k_dual_g(KP<S> p, const S* __restrict__ z, const S* __restrict__ zp,
                                                 const S* __restrict__ eta, S* __restrict__ out) {
+  pdl_enter();
   if (p.skip && *p.skip) return;
   constexpr bool HZ = MODE != DM_PROXG;
   constexpr bool HZP = MODE == DM_DUAL;
@@ -417,6 +420,7 @@ template <typename S, bool DR, int J>
 __global__ void __launch_bounds__(128) k_dual_fused_g(KP<S> p, const S* __restrict__ z, const S* __restrict__ zp,
                                                       const S* __restrict__ eta, S* __restrict__ out,
                                                       const S* __restrict__ dir, double* __restrict__ partials) {
+  pdl_enter();
   if (p.skip && *p.skip) return;
   constexpr int NV = DR ? 3 : 2;   // the rows at q_z = 2 z+ - z, r_z = z - z+ and the direction d_z
   const GenMats<S> G{p};
@@ -644,8 +648,8 @@ static int gen_slots(const KP<S>& p) {
 template <typename S>
 void launch_lstar_gen(const KP<S>& p, int mode, const S* eta, const S* z, S* zo, int grid, cudaStream_t st) {
 #define SPOCK_LG(JJ)                                                                        \
-  if (mode == LS_PREP) k_lstar_g<S, LS_PREP, JJ><<<grid, 128, 0, st>>>(p, eta, z, zo);     \
-  else k_lstar_g<S, LS_APPLY, JJ><<<grid, 128, 0, st>>>(p, eta, z, zo);
+  if (mode == LS_PREP) launch_pdl(k_lstar_g<S, LS_PREP, JJ>, grid, 128, 0, st, p, eta, z, zo);     \
+  else launch_pdl(k_lstar_g<S, LS_APPLY, JJ>, grid, 128, 0, st, p, eta, z, zo);
   switch (gen_slots(p)) {
     case 1: SPOCK_LG(1) break;
     case 3: SPOCK_LG(3) break;
@@ -658,11 +662,11 @@ template <typename S>
 void launch_dual_gen(const KP<S>& p, int mode, bool stats, const S* z, const S* zp, const S* eta, S* out,
                      const S* dir, double* partials, int grid, cudaStream_t st) {
 #define SPOCK_DG(JJ)                                                                                     \
-  if (mode == DM_APPLY_L) k_dual_g<S, DM_APPLY_L, JJ><<<grid, 128, 0, st>>>(p, z, zp, eta, out);         \
-  else if (mode == DM_PROXG) k_dual_g<S, DM_PROXG, JJ><<<grid, 128, 0, st>>>(p, z, zp, eta, out);        \
-  else if (!stats) k_dual_g<S, DM_DUAL, JJ><<<grid, 128, 0, st>>>(p, z, zp, eta, out);                   \
-  else if (dir) k_dual_fused_g<S, true, JJ><<<grid, 128, 0, st>>>(p, z, zp, eta, out, dir, partials);    \
-  else k_dual_fused_g<S, false, JJ><<<grid, 128, 0, st>>>(p, z, zp, eta, out, dir, partials);
+  if (mode == DM_APPLY_L) launch_pdl(k_dual_g<S, DM_APPLY_L, JJ>, grid, 128, 0, st, p, z, zp, eta, out);         \
+  else if (mode == DM_PROXG) launch_pdl(k_dual_g<S, DM_PROXG, JJ>, grid, 128, 0, st, p, z, zp, eta, out);        \
+  else if (!stats) launch_pdl(k_dual_g<S, DM_DUAL, JJ>, grid, 128, 0, st, p, z, zp, eta, out);                   \
+  else if (dir) launch_pdl(k_dual_fused_g<S, true, JJ>, grid, 128, 0, st, p, z, zp, eta, out, dir, partials);    \
+  else launch_pdl(k_dual_fused_g<S, false, JJ>, grid, 128, 0, st, p, z, zp, eta, out, dir, partials);
   switch (gen_slots(p)) {
     case 1: SPOCK_DG(1) break;
     case 3: SPOCK_DG(3) break;

@@ -48,6 +48,7 @@
 
 #include "batch.cuh"
 #include "kernels.cuh"
+#include "launch.cuh"
 #include "spock_internal.h"
 #include "tma.cuh"
 
@@ -184,21 +185,35 @@ struct SeqRing {
   }
 };
 
-// The fetching thread's loop: copies(slot, k, top) starts node k's copies
-// (top: the first node of a sequence); on return nothing is in flight
-// (bounded).
-template <typename F>
-__device__ __forceinline__ void seq_fetch(SeqRing& ring, const int32_t* stage_begin, int t_first, int t_last, int cnt,
-                                          int bid, int nblk, int D, int32_t* err, F copies) {
+// The fetching thread's loop.  fixed(slot, k, above) starts the copies of node
+// k's factors and announces the bytes of all its copies, moving(slot, k, above)
+// those of what earlier kernels write (above: the node before it in the
+// sequence, -1 at the first one).  The factors of the first D nodes are on
+// their way while the previous kernel still runs.  On return nothing is in
+// flight (bounded).
+template <typename F, typename M>
+__device__ __forceinline__ void seq_fetch(SeqRing& ring, const int32_t* skip, const int32_t* stage_begin, int t_first,
+                                          int t_last, int cnt, int bid, int nblk, int D, int32_t* err, F fixed,
+                                          M moving) {
   const int dt = t_first < t_last ? 1 : -1;
-  int slot = 0, issued = 0;
-  for (int ci = bid; ci < cnt && !ring.dead; ci += nblk) {
+  int slot = 0, issued = 0, early = 0;
+  for (int ci = bid; ci < cnt && early < D; ci += nblk)
+    for (int t = t_first; early < D; t += dt) {
+      fixed(early, stage_begin[t] + ci, t == t_first ? -1 : stage_begin[t - dt] + ci);
+      ++early;
+      if (t == t_last) break;
+    }
+  pdl_enter();
+  bool done = false;   // the solve has finished: only complete what has been announced
+  for (int ci = bid; ci < cnt && !ring.dead && !done; ci += nblk) {
     for (int t = t_first;; t += dt) {
-      const int k = stage_begin[t] + ci;
-      if (issued >= D) ring.wait(ring.empty, slot, err);
-      if (ring.dead) break;
+      const int k = stage_begin[t] + ci, above = t == t_first ? -1 : stage_begin[t - dt] + ci;
+      if (issued == early && skip && *skip) done = true;
+      if (issued >= D && !done) ring.wait(ring.empty, slot, err);
+      if (ring.dead || done) break;
       fence_proxy_async();
-      copies(slot, k, t == t_first ? -1 : stage_begin[t - dt] + ci);
+      if (issued >= early) fixed(slot, k, above);
+      moving(slot, k, above);
       ++issued;
       if (++slot == D) slot = 0;
       if (t == t_last) break;
@@ -214,7 +229,6 @@ __device__ __forceinline__ void seq_fetch(SeqRing& ring, const int32_t* stage_be
 // every nblk-th.
 template <typename S>
 __device__ __forceinline__ void bwd_seq_body(const KP<S>& p, int t_hi, int t_lo, int bid, int nblk, int D) {
-  if (p.skip && *p.skip) return;
   using Mat = typename Fx<S>::Mat;
   using Vec = typename Fx<S>::Vec;
   using Acc = typename Fx<S>::Acc;
@@ -242,20 +256,25 @@ __device__ __forceinline__ void bwd_seq_body(const KP<S>& p, int t_hi, int t_lo,
   if (tid >= T) {
     if (tid > T) return;
     const uint32_t xB = p.xs * (uint32_t)sizeof(S), uB = p.us * (uint32_t)sizeof(S);
-    seq_fetch(ring, p.stage_begin, t_hi, t_lo, cnt, bid, nblk, D, p.err, [&](int slot, int k, int) {
-      const bool leaf = k >= p.nl;
-      unsigned char* dst = smem + slot * Ly.item;
-      uint64_t* bar = &ring.full[slot];
-      mbar_expect_tx(bar, xB + (leaf ? 0u : p.nbB + uB) + (k > 0 ? p.gbB : 0u));
-      if (!leaf) {
-        bulk_g2s(dst + p.gbB, p.pNB + (size_t)k * p.nbB, p.nbB, bar);
-        bulk_g2s(dst + p.gbB + p.nbB + xB, p.ubar + (size_t)k * p.us, uB, bar);
-      }
-      bulk_g2s(dst + p.gbB + p.nbB, p.xbar + (size_t)k * p.xs, xB, bar);
-      if (k > 0) bulk_g2s(dst, p.pGb + (size_t)(k - 1) * p.gbB, p.gbB, bar);
-    });
+    seq_fetch(
+        ring, p.skip, p.stage_begin, t_hi, t_lo, cnt, bid, nblk, D, p.err,
+        [&](int slot, int k, int) {
+          const bool leaf = k >= p.nl;
+          unsigned char* dst = smem + slot * Ly.item;
+          uint64_t* bar = &ring.full[slot];
+          mbar_expect_tx(bar, xB + (leaf ? 0u : p.nbB + uB) + (k > 0 ? p.gbB : 0u));
+          if (!leaf) bulk_g2s(dst + p.gbB, p.pNB + (size_t)k * p.nbB, p.nbB, bar);
+          if (k > 0) bulk_g2s(dst, p.pGb + (size_t)(k - 1) * p.gbB, p.gbB, bar);
+        },
+        [&](int slot, int k, int) {
+          unsigned char* dst = smem + slot * Ly.item + p.gbB + p.nbB;
+          if (k < p.nl) bulk_g2s(dst + xB, p.ubar + (size_t)k * p.us, uB, &ring.full[slot]);
+          bulk_g2s(dst, p.xbar + (size_t)k * p.xs, xB, &ring.full[slot]);
+        });
     return;
   }
+  pdl_enter();
+  if (p.skip && *p.skip) return;
   Vec* const A = reinterpret_cast<Vec*>(smem + D * Ly.item);               // (g; -ubar), 4-entry aligned halves
   Vec* const B = reinterpret_cast<Vec*>(smem + D * Ly.item + Ly.vecA);     // q
   Acc* const part = reinterpret_cast<Acc*>(smem + D * Ly.item + Ly.vecA + Ly.vecB);
@@ -339,7 +358,6 @@ __device__ __forceinline__ void bwd_seq_body(const KP<S>& p, int t_hi, int t_lo,
 template <typename S>
 __device__ __forceinline__ void fwd_seq_body(const KP<S>& p, int t_lo, int t_hi, S* __restrict__ zo, int bid,
                                              int nblk, int D) {
-  if (p.skip && *p.skip) return;
   using Mat = typename Fx<S>::Mat;
   using Vec = typename Fx<S>::Vec;
   using Acc = typename Fx<S>::Acc;
@@ -366,19 +384,25 @@ __device__ __forceinline__ void fwd_seq_body(const KP<S>& p, int t_lo, int t_hi,
   if (tid >= T) {
     if (tid > T) return;
     const uint32_t uB = p.us * (uint32_t)sizeof(S);
-    seq_fetch(ring, p.stage_begin, t_lo, t_hi, cnt, bid, nblk, D, p.err, [&](int slot, int k, int above) {
-      const bool leaf = k >= p.nl;
-      const int par = above < 0 ? p.parent[k] : above;
-      const bool first = above >= 0 || k == 1 || p.parent[k - 1] != par;   // k is its parent's first child
-      unsigned char* dst = smem + slot * Ly.item;
-      uint64_t* bar = &ring.full[slot];
-      mbar_expect_tx(bar, p.gfB + (first ? p.ktB : 0u) + (leaf ? 0u : uB));
-      bulk_g2s(dst, p.pGf + (size_t)(k - 1) * p.gfB, p.gfB, bar);
-      if (first) bulk_g2s(dst + p.gfB, p.pKt + (size_t)par * p.ktB, p.ktB, bar);
-      if (!leaf) bulk_g2s(dst + p.gfB + p.ktB, p.d + (size_t)k * p.us, uB, bar);
-    });
+    seq_fetch(
+        ring, p.skip, p.stage_begin, t_lo, t_hi, cnt, bid, nblk, D, p.err,
+        [&](int slot, int k, int above) {
+          const int par = above < 0 ? p.parent[k] : above;
+          const bool first = above >= 0 || k == 1 || p.parent[k - 1] != par;   // k is its parent's first child
+          unsigned char* dst = smem + slot * Ly.item;
+          uint64_t* bar = &ring.full[slot];
+          mbar_expect_tx(bar, p.gfB + (first ? p.ktB : 0u) + (k < p.nl ? uB : 0u));
+          bulk_g2s(dst, p.pGf + (size_t)(k - 1) * p.gfB, p.gfB, bar);
+          if (first) bulk_g2s(dst + p.gfB, p.pKt + (size_t)par * p.ktB, p.ktB, bar);
+        },
+        [&](int slot, int k, int) {
+          if (k < p.nl)
+            bulk_g2s(smem + slot * Ly.item + p.gfB + p.ktB, p.d + (size_t)k * p.us, uB, &ring.full[slot]);
+        });
     return;
   }
+  pdl_enter();
+  if (p.skip && *p.skip) return;
   Vec* W = reinterpret_cast<Vec*>(smem + D * Ly.item);              // (x; d) of the parent
   Vec* Y = reinterpret_cast<Vec*>(smem + D * Ly.item + Ly.vecA);    // (x; d) of the node
   Acc* const part = reinterpret_cast<Acc*>(smem + D * Ly.item + Ly.vecA + Ly.vecB);
@@ -555,7 +579,7 @@ int launch_bwd_seq(const KP<S>& p, int t_hi, int t_lo, int cnt, cudaStream_t st)
   const SeqShape s = seq_shape(p, cnt, t_hi - t_lo + 1, [](const KP<S>& q, int T) { return seq_layout_bwd(q, T); });
   static std::atomic<uint64_t> done{0};
   allow_smem(k_bwd_seq<S>, done);
-  k_bwd_seq<S><<<s.grid, s.T + 32, s.bytes, st>>>(p, t_hi, t_lo, s.D);
+  launch_pdl(k_bwd_seq<S>, s.grid, s.T + 32, s.bytes, st, p, t_hi, t_lo, s.D);
   return 1;
 }
 template <typename S>
@@ -563,7 +587,7 @@ int launch_fwd_seq(const KP<S>& p, int t_lo, int t_hi, int cnt, S* zo, cudaStrea
   const SeqShape s = seq_shape(p, cnt, t_hi - t_lo + 1, [](const KP<S>& q, int T) { return seq_layout_fwd(q, T); });
   static std::atomic<uint64_t> done{0};
   allow_smem(k_fwd_seq<S>, done);
-  k_fwd_seq<S><<<s.grid, s.T + 32, s.bytes, st>>>(p, t_lo, t_hi, zo, s.D);
+  launch_pdl(k_fwd_seq<S>, s.grid, s.T + 32, s.bytes, st, p, t_lo, t_hi, zo, s.D);
   return 1;
 }
 
@@ -589,11 +613,11 @@ void launch_seq_b(int which, const BInst<S>* bi, const BMap& m, int nblocks, con
   if (which <= 1) {
     static std::atomic<uint64_t> done{0};
     allow_smem(k_bwd_seq_b<S>, done);
-    k_bwd_seq_b<S><<<nblocks, sh.T + 32, sh.bytes_bwd, st>>>(bi, m);
+    launch_pdl(k_bwd_seq_b<S>, nblocks, sh.T + 32, sh.bytes_bwd, st, bi, m);
   } else {
     static std::atomic<uint64_t> done{0};
     allow_smem(k_fwd_seq_b<S>, done);
-    k_fwd_seq_b<S><<<nblocks, sh.T + 32, sh.bytes_fwd, st>>>(bi, m);
+    launch_pdl(k_fwd_seq_b<S>, nblocks, sh.T + 32, sh.bytes_fwd, st, bi, m);
   }
 }
 

@@ -15,6 +15,7 @@
 
 #include "batch.cuh"
 #include "kernels.cuh"
+#include "launch.cuh"
 #include "ops_body.cuh"
 #include "rounds_body.cuh"
 #include "supermann.cuh"
@@ -23,6 +24,7 @@ namespace spock {
 
 __global__ void __launch_bounds__(256) k_round_decide(SmState* st, const double* __restrict__ pd, int nd,
                                                       double* stats_t, int32_t* trace) {
+  pdl_enter();
   reduce_stats_body(pd, nd, nullptr, 0, stats_t, &st->done);
   __syncthreads();
   if (threadIdx.x == 0) round_decide_body(st, stats_t, trace);
@@ -33,6 +35,7 @@ __global__ void __launch_bounds__(256, 4) k_round_commit(SmState* st, S* __restr
                                                          const S* __restrict__ Vt, const S* __restrict__ TVt,
                                                          S* __restrict__ MR, S* __restrict__ D, int64_t n,
                                                          int64_t ld, double* __restrict__ partials) {
+  pdl_enter();
   round_commit_body<S, MEM>(st, V, TV, Vt, TVt, MR, D, n, ld, partials, blockIdx.x, gridDim.x);
   if (MEM > 0) round_commit_last(st, partials, gridDim.x);
 }
@@ -42,6 +45,7 @@ __global__ void __launch_bounds__(256) k_round_point(const SmState* __restrict__
                                                      const S* __restrict__ TV, S* __restrict__ Vt,
                                                      const S* __restrict__ TVt, S* __restrict__ d,
                                                      const S* __restrict__ D, int64_t n, int64_t ld) {
+  pdl_enter();
   round_point_body<S, MEM>(st, V, TV, Vt, TVt, d, D, n, ld, blockIdx.x, gridDim.x);
 }
 
@@ -50,6 +54,7 @@ __global__ void __launch_bounds__(256) k_round_point(const SmState* __restrict__
 // ---------------------------------------------------------------------------
 template <typename S>
 __global__ void __launch_bounds__(256) k_round_decide_b(const BInst<S>* __restrict__ bi) {
+  pdl_enter();
   const BInst<S>& b = bi[blockIdx.x];
   reduce_stats_body(b.pd, b.nb_node, nullptr, 0, b.stats, b.kp.skip);
   __syncthreads();
@@ -57,6 +62,7 @@ __global__ void __launch_bounds__(256) k_round_decide_b(const BInst<S>* __restri
 }
 template <typename S, int MEM>
 __global__ void __launch_bounds__(256, 4) k_round_commit_b(const BInst<S>* __restrict__ bi, BMap m) {
+  pdl_enter();
   const int i = m.inst[blockIdx.x];
   const BInst<S>& b = bi[i];
   round_commit_body<S, MEM>(b.st, b.V, b.TV, b.Vt, b.TVt, b.MR, b.D, b.n_v, b.ld, b.paa,
@@ -65,6 +71,7 @@ __global__ void __launch_bounds__(256, 4) k_round_commit_b(const BInst<S>* __res
 }
 template <typename S, int MEM>
 __global__ void __launch_bounds__(256) k_round_point_b(const BInst<S>* __restrict__ bi, BMap m) {
+  pdl_enter();
   const int i = m.inst[blockIdx.x];
   const BInst<S>& b = bi[i];
   round_point_body<S, MEM>(b.st, b.V, b.TV, b.Vt, b.TVt, b.d, b.D, b.n_v, b.ld, blockIdx.x - m.base[i],
@@ -72,7 +79,7 @@ __global__ void __launch_bounds__(256) k_round_point_b(const BInst<S>* __restric
 }
 
 void launch_round_decide(SmState* st, const double* pd, int nd, double* stats_t, int32_t* trace, cudaStream_t s) {
-  k_round_decide<<<1, 256, 0, s>>>(st, pd, nd, stats_t, trace);
+  launch_pdl(k_round_decide, 1, 256, 0, s, st, pd, nd, stats_t, trace);
 }
 
 template <typename S>
@@ -80,7 +87,7 @@ void launch_round_commit(SmState* st, S* V, S* TV, const S* Vt, const S* TVt, S*
                          int64_t n, int64_t ld, int mem, double* partials, int grid, cudaStream_t s) {
   switch (mem) {
 #define SPOCK_RC(M) \
-  case M: k_round_commit<S, M><<<grid, 256, 0, s>>>(st, V, TV, Vt, TVt, MR, D, n, ld, partials); break;
+  case M: launch_pdl(k_round_commit<S, M>, grid, 256, 0, s, st, V, TV, Vt, TVt, MR, D, n, ld, partials); break;
     SPOCK_RC(0) SPOCK_RC(1) SPOCK_RC(2) SPOCK_RC(3) SPOCK_RC(4) SPOCK_RC(5) SPOCK_RC(6) SPOCK_RC(7) SPOCK_RC(8)
     SPOCK_RC(9) SPOCK_RC(10) SPOCK_RC(11) SPOCK_RC(12) SPOCK_RC(13) SPOCK_RC(14) SPOCK_RC(15) SPOCK_RC(16)
 #undef SPOCK_RC
@@ -91,7 +98,7 @@ template <typename S>
 void launch_round_point(SmState* st, const S* V, const S* TV, S* Vt, const S* TVt, S* d, const S* D, int64_t n,
                         int64_t ld, int mem, int grid, cudaStream_t s) {
   switch (mem) {
-#define SPOCK_RP(M) case M: k_round_point<S, M><<<grid, 256, 0, s>>>(st, V, TV, Vt, TVt, d, D, n, ld); break;
+#define SPOCK_RP(M) case M: launch_pdl(k_round_point<S, M>, grid, 256, 0, s, st, V, TV, Vt, TVt, d, D, n, ld); break;
     SPOCK_RP(0) SPOCK_RP(1) SPOCK_RP(2) SPOCK_RP(3) SPOCK_RP(4) SPOCK_RP(5) SPOCK_RP(6) SPOCK_RP(7) SPOCK_RP(8)
     SPOCK_RP(9) SPOCK_RP(10) SPOCK_RP(11) SPOCK_RP(12) SPOCK_RP(13) SPOCK_RP(14) SPOCK_RP(15) SPOCK_RP(16)
 #undef SPOCK_RP
@@ -101,12 +108,12 @@ void launch_round_point(SmState* st, const S* V, const S* TV, S* Vt, const S* TV
 
 template <typename S>
 void launch_round_decide_b(const BInst<S>* bi, int n_inst, cudaStream_t st) {
-  k_round_decide_b<S><<<n_inst, 256, 0, st>>>(bi);
+  launch_pdl(k_round_decide_b<S>, n_inst, 256, 0, st, bi);
 }
 template <typename S>
 void launch_round_commit_b(const BInst<S>* bi, const BMap& m, int nblocks, int mem, cudaStream_t st) {
   switch (mem) {
-#define SPOCK_RC(M) case M: k_round_commit_b<S, M><<<nblocks, 256, 0, st>>>(bi, m); break;
+#define SPOCK_RC(M) case M: launch_pdl(k_round_commit_b<S, M>, nblocks, 256, 0, st, bi, m); break;
     SPOCK_RC(0) SPOCK_RC(1) SPOCK_RC(2) SPOCK_RC(3) SPOCK_RC(4) SPOCK_RC(5) SPOCK_RC(6) SPOCK_RC(7) SPOCK_RC(8)
     SPOCK_RC(9) SPOCK_RC(10) SPOCK_RC(11) SPOCK_RC(12) SPOCK_RC(13) SPOCK_RC(14) SPOCK_RC(15) SPOCK_RC(16)
 #undef SPOCK_RC
@@ -116,7 +123,7 @@ void launch_round_commit_b(const BInst<S>* bi, const BMap& m, int nblocks, int m
 template <typename S>
 void launch_round_point_b(const BInst<S>* bi, const BMap& m, int nblocks, int mem, cudaStream_t st) {
   switch (mem) {
-#define SPOCK_RP(M) case M: k_round_point_b<S, M><<<nblocks, 256, 0, st>>>(bi, m); break;
+#define SPOCK_RP(M) case M: launch_pdl(k_round_point_b<S, M>, nblocks, 256, 0, st, bi, m); break;
     SPOCK_RP(0) SPOCK_RP(1) SPOCK_RP(2) SPOCK_RP(3) SPOCK_RP(4) SPOCK_RP(5) SPOCK_RP(6) SPOCK_RP(7) SPOCK_RP(8)
     SPOCK_RP(9) SPOCK_RP(10) SPOCK_RP(11) SPOCK_RP(12) SPOCK_RP(13) SPOCK_RP(14) SPOCK_RP(15) SPOCK_RP(16)
 #undef SPOCK_RP

@@ -15,6 +15,7 @@
 
 #include "batch.cuh"
 #include "kernels.cuh"
+#include "launch.cuh"
 #include "general.h"
 #include "spock_internal.h"
 #include "supermann.cuh"
@@ -425,6 +426,7 @@ static void eval_T(const Ctx& c, const S* v, S* Tv, const S* dir, double* stats,
   const int64_t nz = P.off.n_z;
   const int maxb = sm_count() * 16;
   cudaEvent_t* ev = (ws && ws->prof.on) ? ws->prof.slot() : nullptr;
+  const PlainLaunches plain(ev != nullptr);
   if (ev) record_event(ev[0], c.st);
   launch_prep<S>(kp, v, v + nz, Tv, maxb, c.st);
   if (ev) record_event(ev[1], c.st);
@@ -653,6 +655,7 @@ static int solve_graph(Problem& P, const double* x0_dev, const spock_settings& s
                        int warm, spock_info* info, cudaStream_t user_st, double tol_given, int stall_window,
                        int* final_action_out, bool cta = false) {
   const int mem = std::max(0, std::min<int>(s.memory, kMaxMemory));
+  const PlainLaunches plain(s.profile != 0);   // a kernel after an event record
   Workspace* ws = get_ws_impl<S>(P, mem);
   const DevFactors<S>& f = factors<S>(P);
   const int64_t nz = P.off.n_z, nv = ws->n_v;
