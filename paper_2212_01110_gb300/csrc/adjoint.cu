@@ -16,6 +16,7 @@
 #include <algorithm>
 
 #include "kernels.cuh"
+#include "launch.cuh"
 #include "spock_internal.h"
 
 namespace spock {
@@ -88,6 +89,7 @@ __device__ __forceinline__ void soc_jac_block(const double* __restrict__ wb, con
 template <int J>
 __global__ void __launch_bounds__(128) k_cone_jac(KP<double> p, const double* __restrict__ wbar,
                                                   const double* __restrict__ x, double* __restrict__ out) {
+  pdl_enter();
   const int lane = threadIdx.x & 31;
   const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int nw = (gridDim.x * blockDim.x) >> 5;
@@ -123,6 +125,7 @@ __global__ void __launch_bounds__(128) k_cone_jac(KP<double> p, const double* __
 // out = y + a x
 __global__ void k_axpy(int64_t n, double a, const double* __restrict__ x, const double* __restrict__ y,
                        double* __restrict__ out) {
+  pdl_enter();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     out[i] = y[i] + a * x[i];
 }
@@ -140,6 +143,7 @@ constexpr int kGmresMaxRestart = 128; // basis vectors of one axpy launch
 __global__ void k_jt_residual(int64_t nz, int64_t ne, double alpha, const double* __restrict__ pz,
                               const double* __restrict__ t, const double* __restrict__ q,
                               const double* __restrict__ Lp, const double* __restrict__ x, double* __restrict__ u) {
+  pdl_enter();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nz + ne;
        i += (int64_t)gridDim.x * blockDim.x)
     u[i] = x[i] - (i < nz ? pz[i] - alpha * t[i] : q[i - nz] - alpha * Lp[i - nz]);
@@ -151,6 +155,7 @@ __global__ void k_jt_residual(int64_t nz, int64_t ne, double alpha, const double
 __global__ void __launch_bounds__(256) k_dots(int64_t n, const double* __restrict__ u, const double* __restrict__ V,
                                               int64_t ld, int k, const int* __restrict__ kdev,
                                               double* __restrict__ partials) {
+  pdl_enter();
   if (kdev) k += *kdev;
   __shared__ double red[8][kGmresMaxBasis];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -167,10 +172,13 @@ __global__ void __launch_bounds__(256) k_dots(int64_t n, const double* __restric
         if (j < kc) acc[j] = fma(ui, Vc[(int64_t)j * ld + i], acc[j]);
     }
 #pragma unroll
-    for (int j = 0; j < kGmresMaxBasis; ++j) {
-      if (j < kc) {
-        const double v = warp_sum(acc[j]);
-        if (lane == 0) red[w][j] = v;
+    for (int g = 0; g < kGmresMaxBasis / 8; ++g) {   // eight sums at a time (warp-uniform condition)
+      if (8 * g < kc) {
+        double v[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = acc[8 * g + i];
+        const double t = warp_sum8(v, lane);
+        if ((lane & 3) == 0) red[w][8 * g + warp_sum8_index(lane)] = t;
       }
     }
     __syncthreads();
@@ -183,14 +191,19 @@ __global__ void __launch_bounds__(256) k_dots(int64_t n, const double* __restric
   }
 }
 
-// out[j] = sum_b partials[b][j], j < k (one block, fixed order)
-__global__ void k_dots_reduce(int nblocks, int k, const int* __restrict__ kdev, const double* __restrict__ partials,
-                              double* __restrict__ out) {
+// out[j] = sum_b partials[b][j], j < k (one block, fixed order): a warp per
+// value, lanes over the rows.  (One thread over the 608 rows of a full grid is
+// a chain of 608 FP64 additions: 69 us, three times per Arnoldi step.)
+__global__ void __launch_bounds__(1024) k_dots_reduce(int nblocks, int k, const int* __restrict__ kdev,
+                                                      const double* __restrict__ partials, double* __restrict__ out) {
+  pdl_enter();
   if (kdev) k += *kdev;
-  for (int j = threadIdx.x; j < k; j += blockDim.x) {
+  const int lane = threadIdx.x & 31;
+  for (int j = threadIdx.x >> 5; j < k; j += blockDim.x >> 5) {
     double s = 0.0;
-    for (int b = 0; b < nblocks; ++b) s += partials[(int64_t)b * kGmresMaxRestart + j];
-    out[j] = s;
+    for (int b = lane; b < nblocks; b += 32) s += partials[(int64_t)b * kGmresMaxRestart + j];
+    s = warp_sum(s);
+    if (lane == 0) out[j] = s;
   }
 }
 
@@ -198,6 +211,7 @@ __global__ void k_dots_reduce(int nblocks, int k, const int* __restrict__ kdev, 
 // with kdev, k is *kdev + k)
 __global__ void k_axpy_many(int64_t n, double* __restrict__ u, const double* __restrict__ V, int64_t ld, int k,
                             const int* __restrict__ kdev, const double* __restrict__ h, double sign) {
+  pdl_enter();
   if (kdev) k += *kdev;
   __shared__ double hs[kGmresMaxRestart];
   for (int j = threadIdx.x; j < k; j += blockDim.x) hs[j] = sign * h[j];
@@ -211,6 +225,7 @@ __global__ void k_axpy_many(int64_t n, double* __restrict__ u, const double* __r
 
 // v = a u
 __global__ void k_scale(int64_t n, double a, const double* __restrict__ u, double* __restrict__ v) {
+  pdl_enter();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     v[i] = a * u[i];
 }
@@ -220,6 +235,7 @@ __global__ void k_scale(int64_t n, double a, const double* __restrict__ u, doubl
 __global__ void k_next_basis(int64_t n, const double* __restrict__ u, const double* __restrict__ norm2,
                              const int* __restrict__ kdev, double* __restrict__ V, int64_t ld,
                              double* __restrict__ vin) {
+  pdl_enter();
   const double nn = *norm2;
   const double a = nn > 0.0 ? 1.0 / sqrt(nn) : 0.0;
   double* vk1 = V + (int64_t)(*kdev + 1) * ld;
@@ -230,12 +246,14 @@ __global__ void k_next_basis(int64_t n, const double* __restrict__ u, const doub
   }
 }
 
-__global__ void k_inc(int* kdev) { *kdev += 1; }
+__global__ void k_inc(int* kdev) {
+  pdl_enter(); *kdev += 1; }
 
 // red[0] = max |b - u|, red[1] = max |x| (bit patterns of non-negative
 // doubles), r = b - u written out; b = (g, 0)
 __global__ void k_true_residual(int64_t nz, int64_t ntot, const double* __restrict__ g, const double* __restrict__ u,
                                 const double* __restrict__ x, double* __restrict__ r, unsigned long long* red) {
+  pdl_enter();
   double rmax = 0.0, xmax = 0.0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < ntot; i += (int64_t)gridDim.x * blockDim.x) {
     const double ri = (i < nz ? g[i] : 0.0) - u[i];
@@ -266,6 +284,7 @@ __global__ void __launch_bounds__(128) k_adj_gradients(KP<double> p, const doubl
                                                        const double* __restrict__ lam_env,
                                                        const double* __restrict__ wenv, double* gx0, double* gA,
                                                        double* gB, double* gQ, double* gR, double* gQN) {
+  pdl_enter();
   const int lane = threadIdx.x & 31;
   const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int nw = (gridDim.x * blockDim.x) >> 5;
@@ -312,56 +331,58 @@ void launch_cone_jac(const KP<double>& p, const double* wbar, const double* x, d
                      cudaStream_t st) {
   const int J = (p.nx + p.nu + 2 + 31) / 32;
   switch (J) {
-    case 1: k_cone_jac<1><<<grid, 128, 0, st>>>(p, wbar, x, out); break;
-    case 2: k_cone_jac<2><<<grid, 128, 0, st>>>(p, wbar, x, out); break;
-    case 3: k_cone_jac<3><<<grid, 128, 0, st>>>(p, wbar, x, out); break;
-    case 4: k_cone_jac<4><<<grid, 128, 0, st>>>(p, wbar, x, out); break;
-    default: k_cone_jac<5><<<grid, 128, 0, st>>>(p, wbar, x, out); break;
+    case 1: launch_pdl(k_cone_jac<1>, grid, 128, 0, st, p, wbar, x, out); break;
+    case 2: launch_pdl(k_cone_jac<2>, grid, 128, 0, st, p, wbar, x, out); break;
+    case 3: launch_pdl(k_cone_jac<3>, grid, 128, 0, st, p, wbar, x, out); break;
+    case 4: launch_pdl(k_cone_jac<4>, grid, 128, 0, st, p, wbar, x, out); break;
+    default: launch_pdl(k_cone_jac<5>, grid, 128, 0, st, p, wbar, x, out); break;
   }
 }
 
 void launch_axpy(int64_t n, double a, const double* x, const double* y, double* out, int grid, cudaStream_t st) {
-  k_axpy<<<grid, 256, 0, st>>>(n, a, x, y, out);
+  launch_pdl(k_axpy, grid, 256, 0, st, n, a, x, y, out);
 }
 
 void launch_jt_residual(int64_t nz, int64_t ne, double alpha, const double* pz, const double* t, const double* q,
                         const double* Lp, const double* x, double* u, int grid, cudaStream_t st) {
-  k_jt_residual<<<grid, 256, 0, st>>>(nz, ne, alpha, pz, t, q, Lp, x, u);
+  launch_pdl(k_jt_residual, grid, 256, 0, st, nz, ne, alpha, pz, t, q, Lp, x, u);
 }
 
 // out[j] = u . V_j for j < k (k <= 128; plus *kdev when kdev is given) in
 // two launches; partials holds grid x 128 doubles
 void launch_dots(int64_t n, const double* u, const double* V, int64_t ld, int k, const int* kdev, double* partials,
                  double* out, int grid, cudaStream_t st) {
-  k_dots<<<grid, 256, 0, st>>>(n, u, V, ld, k, kdev, partials);
-  k_dots_reduce<<<1, kGmresMaxRestart, 0, st>>>(grid, k, kdev, partials, out);
+  // at least four entries a thread: fewer rows of partials to add
+  const int g = (int)std::max<int64_t>(1, std::min<int64_t>(grid, (n + 1023) / 1024));
+  launch_pdl(k_dots, g, 256, 0, st, n, u, V, ld, k, kdev, partials);
+  launch_pdl(k_dots_reduce, 1, 1024, 0, st, g, k, kdev, partials, out);
 }
 
 void launch_axpy_many(int64_t n, double* u, const double* V, int64_t ld, int k, const int* kdev, const double* h,
                       double sign, int grid, cudaStream_t st) {
-  k_axpy_many<<<grid, 256, 0, st>>>(n, u, V, ld, k, kdev, h, sign);
+  launch_pdl(k_axpy_many, grid, 256, 0, st, n, u, V, ld, k, kdev, h, sign);
 }
 
 void launch_next_basis(int64_t n, const double* u, const double* norm2, int* kdev, double* V, int64_t ld,
                        double* vin, int grid, cudaStream_t st) {
-  k_next_basis<<<grid, 256, 0, st>>>(n, u, norm2, kdev, V, ld, vin);
-  k_inc<<<1, 1, 0, st>>>(kdev);
+  launch_pdl(k_next_basis, grid, 256, 0, st, n, u, norm2, kdev, V, ld, vin);
+  launch_pdl(k_inc, 1, 1, 0, st, kdev);
 }
 
 void launch_scale(int64_t n, double a, const double* u, double* v, int grid, cudaStream_t st) {
-  k_scale<<<grid, 256, 0, st>>>(n, a, u, v);
+  launch_pdl(k_scale, grid, 256, 0, st, n, a, u, v);
 }
 
 void launch_true_residual(int64_t nz, int64_t ntot, const double* g, const double* u, const double* x, double* r,
                           unsigned long long* red, int grid, cudaStream_t st) {
-  k_true_residual<<<grid, 256, 0, st>>>(nz, ntot, g, u, x, r, red);
+  launch_pdl(k_true_residual, grid, 256, 0, st, nz, ntot, g, u, x, r, red);
 }
 
 void launch_adj_gradients(const KP<double>& p, const double* z, const double* eta, const double* q,
                           const double* pv, const double* lam_mu, const double* negy, const double* lam_env,
                           const double* wenv, double* gx0, double* gA, double* gB, double* gQ, double* gR,
                           double* gQN, int grid, cudaStream_t st) {
-  k_adj_gradients<<<grid, 128, 0, st>>>(p, z, eta, q, pv, lam_mu, negy, lam_env, wenv, gx0, gA, gB, gQ, gR, gQN);
+  launch_pdl(k_adj_gradients, grid, 128, 0, st, p, z, eta, q, pv, lam_mu, negy, lam_env, wenv, gx0, gA, gB, gQ, gR, gQN);
 }
 
 }  // namespace spock

@@ -14,64 +14,30 @@
 // [Abar^c | B^c] blocks followed by a K^T product.  Then
 //   dV/dx0 = -lambda^0, dV/dA^c = -lambda^c x^anc(c)T, dV/dB^c = -lambda^c u^anc(c)T,
 //   dV/dQ^c_kk = eta*_{c,Qx,k} x^anc_k / (2 sqrt Q^c_kk)  (likewise R, Q_N).
+#include <algorithm>
+#include <vector>
+
 #include "kernels.cuh"
+#include "launch.cuh"
 #include "spock_internal.h"
 
 namespace spock {
 
-// lambda for the nonleaf nodes of stage t (warp per node); lam has stride xs.
-template <typename S, int SL>
-__global__ void __launch_bounds__(128) k_lambda_stage(KP<S> p, int t, const S* __restrict__ w, S* __restrict__ lam) {
-  __shared__ S lv[kWarpsPerBlock][kVecPad];
-  __shared__ S hv[kWarpsPerBlock][kVecPad];
-  const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
-  const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-  const int nx = p.nx, nu = p.nu, ncol = nx + nu;
-  const int b0 = p.stage_begin[t], cnt = p.stage_begin[t + 1] - b0;
-  S* lc = lv[wl];
-  S* hs = hv[wl];
-  for (int idx = gw; idx < cnt; idx += nw) {
-    const int k = b0 + idx;
-    const NodeDesc D = p.desc[k];
-    S h[SL];
-#pragma unroll
-    for (int s = 0; s < SL; ++s) h[s] = S(0);
-    for (int j = 0; j < D.m; ++j) {
-      const int c = D.c0 + j;
-      if (c >= p.nl) {
-        const int64_t zxc = p.desc[c].zx;
-        for (int r = lane; r < nx; r += 32) lc[r] = -w[zxc + r];
-      } else {
-        for (int r = lane; r < nx; r += 32) lc[r] = lam[(int64_t)c * p.xs + r];
-      }
-      __syncwarp();
-      const S* G = p.Gb + (int64_t)(c - 1) * p.gstride;
-      for (int r = 0; r < nx; ++r) {
-        const S lr = lc[r];
-#pragma unroll
-        for (int s = 0; s < SL; ++s) {
-          const int col = 32 * s + lane;
-          if (col < ncol) h[s] += G[(int64_t)r * ncol + col] * lr;
-        }
-      }
-      __syncwarp();
-    }
-#pragma unroll
-    for (int s = 0; s < SL; ++s) {
-      const int col = 32 * s + lane;
-      if (col < ncol) hs[col] = h[s];
-    }
-    __syncwarp();
-    const S* Km = p.NB + (int64_t)k * p.nbstride;  // K: nu x nx
-    for (int r = lane; r < nx; r += 32) {
-      S acc = hs[r] - w[D.zx + r];
-      for (int b = 0; b < nu; ++b) acc -= Km[b * nx + r] * hs[nx + b];
-      lam[(int64_t)k * p.xs + r] = acc;
-    }
-    __syncwarp();
+// The states' part of w in the order and stride of the Riccati scratch (what
+// the sequence kernels fetch): wx[k] = w_x^k.
+template <typename S>
+__global__ void __launch_bounds__(256) k_gather_x(KP<S> p, const S* __restrict__ w, S* __restrict__ wx) {
+  pdl_enter();
+  const int64_t total = (int64_t)p.n * p.nx;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t k = i / p.nx, r = i % p.nx;
+    wx[k * p.xs + r] = w[p.zx[k] + r];
   }
 }
+
+// riccati_seq.cu: the recursion of the multipliers
+template <typename S>
+int launch_lambda_seq(const KP<S>& p, int t_hi, int t_lo, int cnt, S* lam, cudaStream_t st);
 
 // Gradients (FP64 outputs in the caller's node numbering), warp per node.
 template <typename S>
@@ -79,6 +45,7 @@ __global__ void __launch_bounds__(128) k_gradients(KP<S> p, const S* __restrict_
                                                    const S* __restrict__ w, const S* __restrict__ lam,
                                                    double* gx0, double* gA, double* gB, double* gQ, double* gR,
                                                    double* gQN) {
+  pdl_enter();
   const int lane = threadIdx.x & 31;
   const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int nw = (gridDim.x * blockDim.x) >> 5;
@@ -120,23 +87,20 @@ __global__ void __launch_bounds__(128) k_gradients(KP<S> p, const S* __restrict_
 
 // Multipliers of the dynamics for a right-hand side -w_1: the solution of
 // G^T lambda = -w_{z_1} by the tree recursion above (leaves lambda = -w_x,
-// not stored); lam [nonleaf][xs].
+// not stored); lam [nonleaf][xs].  The recursion is the backward Riccati step
+// with q = lambda, xbar = w_x, ubar = h_u and g = 0 (riccati_seq.cu), one
+// launch for the chains and one per branching stage; it uses the Riccati
+// scratch (xbar, hb).
 template <typename S>
 int launch_lambda(const KP<S>& p, const std::vector<int32_t>& stage_begin, const S* w, S* lam, int max_blocks,
                   cudaStream_t st) {
-  const int sl = (p.nx + p.nu + 31) / 32;
-  int launches = 0;
-  for (int t = p.N - 1; t >= 0; --t) {
-    const int cnt = stage_begin[t + 1] - stage_begin[t];
-    const int grid = std::max(1, std::min((cnt + kWarpsPerBlock - 1) / kWarpsPerBlock, max_blocks));
-    switch (sl) {
-      case 1: k_lambda_stage<S, 1><<<grid, 128, 0, st>>>(p, t, w, lam); break;
-      case 2: k_lambda_stage<S, 2><<<grid, 128, 0, st>>>(p, t, w, lam); break;
-      case 3: k_lambda_stage<S, 3><<<grid, 128, 0, st>>>(p, t, w, lam); break;
-      default: k_lambda_stage<S, 4><<<grid, 128, 0, st>>>(p, t, w, lam); break;
-    }
-    ++launches;
-  }
+  const int64_t total = (int64_t)p.n * p.nx;
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((total + 255) / 256, max_blocks));
+  launch_pdl(k_gather_x<S>, grid, 256, 0, st, p, w, p.xbar);
+  auto cnt = [&](int t) { return (int)(stage_begin[t + 1] - stage_begin[t]); };
+  const int cs = p.chain_stage;
+  int launches = 1 + launch_lambda_seq<S>(p, p.N, cs, cnt(cs), lam, st);
+  for (int t = cs - 1; t >= 0; --t) launches += launch_lambda_seq<S>(p, t, t, cnt(t), lam, st);
   return launches;
 }
 template int launch_lambda<double>(const KP<double>&, const std::vector<int32_t>&, const double*, double*, int,
@@ -150,7 +114,7 @@ int launch_gradient(const KP<S>& p, const std::vector<int32_t>& stage_begin, con
                     cudaStream_t st) {
   const int launches = launch_lambda<S>(p, stage_begin, w, lam, max_blocks, st);
   const int grid = std::max(1, std::min((p.n + kWarpsPerBlock - 1) / kWarpsPerBlock, max_blocks));
-  k_gradients<S><<<grid, 128, 0, st>>>(p, z, eta, w, lam, gx0, gA, gB, gQ, gR, gQN);
+  launch_pdl(k_gradients<S>, grid, 128, 0, st, p, z, eta, w, lam, gx0, gA, gB, gQ, gR, gQN);
   return launches + 1;
 }
 

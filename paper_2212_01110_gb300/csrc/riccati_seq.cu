@@ -226,9 +226,12 @@ __device__ __forceinline__ void seq_fetch(SeqRing& ring, const int32_t* skip, co
 }
 
 // Sequences from stage t_hi down to t_lo, of which block bid of nblk takes
-// every nblk-th.
-template <typename S>
-__device__ __forceinline__ void bwd_seq_body(const KP<S>& p, int t_hi, int t_lo, int bid, int nblk, int D) {
+// every nblk-th.  LAM: the recursion of the multipliers (grad.cu), lambda^k =
+// h_x - xbar^k - K^T h_u -- q with g = 0 and ubar = h_u -- into lam instead of
+// d.
+template <typename S, bool LAM>
+__device__ __forceinline__ void bwd_seq_body(const KP<S>& p, int t_hi, int t_lo, int bid, int nblk, int D,
+                                             S* lam = nullptr) {
   using Mat = typename Fx<S>::Mat;
   using Vec = typename Fx<S>::Vec;
   using Acc = typename Fx<S>::Acc;
@@ -309,8 +312,8 @@ __device__ __forceinline__ void bwd_seq_body(const KP<S>& p, int t_hi, int t_lo,
       if (leaf) {
         if (inx) q = -xb[ex];
       } else {
-        const S u = inu ? (xb + p.xs)[tid] : S(0);
-        const S g = inu ? u - h : S(0);
+        const S u = inu ? (LAM ? h : (xb + p.xs)[tid]) : S(0);
+        const S g = !LAM && inu ? u - h : S(0);
         const S base = inx ? h - xb[ex] : S(0);
         const uint32_t kg = seq_kmax<S>(inu ? max(Fx<S>::key(g), Fx<S>::key(u)) : 0u, nu, kword, T);
         if (inu) {
@@ -330,8 +333,12 @@ __device__ __forceinline__ void bwd_seq_body(const KP<S>& p, int t_hi, int t_lo,
         if (own) {
           const int* xn_ = reinterpret_cast<const int*>(it + p.gbB + (nu * ncol + nu * nx) * MB);
           const S v = Fx<S>::value(acc, FX ? Fx<S>::vec_exp(kgs) + xn_[mc] : 0);
-          if (inu) p.d[(int64_t)k * p.us + tid] = v;
-          else q = base + v;
+          if (inx) q = base + v;
+          if (LAM) {
+            if (inx) lam[(int64_t)k * p.xs + ex] = q;
+          } else if (inu) {
+            p.d[(int64_t)k * p.us + tid] = v;
+          }
         }
       }
       if (k > 0) {
@@ -474,7 +481,11 @@ __device__ __forceinline__ void fwd_seq_body(const KP<S>& p, int t_lo, int t_hi,
 
 template <typename S>
 __global__ void __launch_bounds__(kMaxSeqThreads + 32, 1) k_bwd_seq(KP<S> p, int t_hi, int t_lo, int D) {
-  bwd_seq_body<S>(p, t_hi, t_lo, blockIdx.x, gridDim.x, D);
+  bwd_seq_body<S, false>(p, t_hi, t_lo, blockIdx.x, gridDim.x, D);
+}
+template <typename S>
+__global__ void __launch_bounds__(kMaxSeqThreads + 32, 1) k_lambda_seq(KP<S> p, int t_hi, int t_lo, S* lam, int D) {
+  bwd_seq_body<S, true>(p, t_hi, t_lo, blockIdx.x, gridDim.x, D, lam);
 }
 template <typename S>
 __global__ void __launch_bounds__(kMaxSeqThreads + 32, 1) k_fwd_seq(KP<S> p, int t_lo, int t_hi, S* __restrict__ zo,
@@ -488,7 +499,7 @@ template <typename S>
 __global__ void __launch_bounds__(kMaxSeqThreads + 32, 1) k_bwd_seq_b(const BInst<S>* __restrict__ bi, BMap m) {
   const int i = m.inst[blockIdx.x], t = m.stage[i];
   const KP<S> p = bi[i].kp;
-  bwd_seq_body<S>(p, t < 0 ? p.N : t, t < 0 ? p.chain_stage : t, blockIdx.x - m.base[i], m.cnt[i], 1);
+  bwd_seq_body<S, false>(p, t < 0 ? p.N : t, t < 0 ? p.chain_stage : t, blockIdx.x - m.base[i], m.cnt[i], 1);
 }
 template <typename S>
 __global__ void __launch_bounds__(kMaxSeqThreads + 32, 1) k_fwd_seq_b(const BInst<S>* __restrict__ bi, BMap m) {
@@ -583,6 +594,14 @@ int launch_bwd_seq(const KP<S>& p, int t_hi, int t_lo, int cnt, cudaStream_t st)
   return 1;
 }
 template <typename S>
+int launch_lambda_seq(const KP<S>& p, int t_hi, int t_lo, int cnt, S* lam, cudaStream_t st) {
+  const SeqShape s = seq_shape(p, cnt, t_hi - t_lo + 1, [](const KP<S>& q, int T) { return seq_layout_bwd(q, T); });
+  static std::atomic<uint64_t> done{0};
+  allow_smem(k_lambda_seq<S>, done);
+  launch_pdl(k_lambda_seq<S>, s.grid, s.T + 32, s.bytes, st, p, t_hi, t_lo, lam, s.D);
+  return 1;
+}
+template <typename S>
 int launch_fwd_seq(const KP<S>& p, int t_lo, int t_hi, int cnt, S* zo, cudaStream_t st) {
   const SeqShape s = seq_shape(p, cnt, t_hi - t_lo + 1, [](const KP<S>& q, int T) { return seq_layout_fwd(q, T); });
   static std::atomic<uint64_t> done{0};
@@ -623,6 +642,7 @@ void launch_seq_b(int which, const BInst<S>* bi, const BMap& m, int nblocks, con
 
 #define SPOCK_SEQ_INST(S)                                                                            \
   template int launch_bwd_seq<S>(const KP<S>&, int, int, int, cudaStream_t);                         \
+  template int launch_lambda_seq<S>(const KP<S>&, int, int, int, S*, cudaStream_t);                  \
   template int launch_fwd_seq<S>(const KP<S>&, int, int, int, S*, cudaStream_t);                     \
   template bool seq_batch_shape<S>(const std::vector<KP<S>>&, SeqBatchShape&);                       \
   template void launch_seq_b<S>(int, const BInst<S>*, const BMap&, int, const SeqBatchShape&, cudaStream_t);
