@@ -2,6 +2,7 @@
 // evaluation of T as a sequence of kernel launches, the driver loop of
 // Algorithm 3 whose decisions are taken on the device (supermann.cu), the
 // vanilla CP loop and the C ABI of include/spock.h.
+#include <atomic>
 #include <chrono>
 #include <cstdlib>
 #include <cmath>
@@ -76,10 +77,17 @@ int guarded(F&& f) {
 
 // A kernel whose bounded wait on a bulk copy gave up sets *P.err; report it
 // (and clear the flag) after the work on `st` has completed.
-static void check_device_flag(Problem& P, cudaStream_t st) {
+// The copy waits for the stream: callers need not synchronise before it.
+// copied: the flag, if the caller has copied it along with its results and
+// synchronised.
+static void check_device_flag(Problem& P, cudaStream_t st, const int32_t* copied = nullptr) {
   int32_t h = 0;
-  CUDA_TRY(cudaMemcpyAsync(&h, P.err, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-  CUDA_TRY(cudaStreamSynchronize(st));
+  if (copied) {
+    h = *copied;
+  } else {
+    CUDA_TRY(cudaMemcpyAsync(&h, P.err, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+    CUDA_TRY(cudaStreamSynchronize(st));
+  }
   if (h) {
     CUDA_TRY(cudaMemsetAsync(P.err, 0, sizeof(int32_t), st));
     CUDA_TRY(cudaStreamSynchronize(st));
@@ -167,13 +175,15 @@ struct Workspace {
   cudaGraphExec_t gexec = nullptr;
   double g_alpha = 0.0;
   int g_trace = -1, g_launches_per_round = 0;
-  int32_t* h_done = nullptr;  // pinned
+  int32_t* h_done = nullptr;  // pinned: done and rounds, [2] the problem's error flag
+  SmState* h_state = nullptr; // pinned: the state at the end of a solve; its statistics also for CP steps
   void* cta_bi = nullptr;      // instance view of the single-block solve (device)
   std::vector<void*> allocs;
   ~Workspace() {
     if (gexec) cudaGraphExecDestroy(gexec);
     if (stream) cudaStreamDestroy(stream);
     if (h_done) cudaFreeHost(h_done);
+    if (h_state) cudaFreeHost(h_state);
     for (void* p : allocs) cudaFree(p);
     if (h_action) cudaFreeHost(h_action);
     if (e0) cudaEventDestroy(e0);
@@ -195,10 +205,17 @@ Problem::~Problem() {
 }
 
 static int sm_count() {
-  int dev = 0, n = 0;
+  static std::atomic<int> cached[64];   // per device
+  int dev = 0;
   cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-  return n > 0 ? n : 132;
+  std::atomic<int>& c = cached[dev & 63];
+  int n = c.load(std::memory_order_relaxed);
+  if (n == 0) {
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    n = n > 0 ? n : 132;
+    c.store(n, std::memory_order_relaxed);
+  }
+  return n;
 }
 
 template <typename S>
@@ -244,6 +261,7 @@ static Workspace* get_ws_impl(Problem& P, int mem) {
     ws->st = (SmState*)ws->alloc(sizeof(SmState));
     CUDA_TRY(cudaMallocHost(&ws->h_action, sizeof(int32_t) * 4));
     CUDA_TRY(cudaMallocHost(&ws->h_done, sizeof(int32_t) * 4));
+    CUDA_TRY(cudaMallocHost(&ws->h_state, sizeof(SmState)));
     CUDA_TRY(cudaStreamCreateWithFlags(&ws->stream, cudaStreamNonBlocking));
     CUDA_TRY(cudaEventCreate(&ws->e0));
     CUDA_TRY(cudaEventCreate(&ws->e1));
@@ -732,8 +750,8 @@ static int solve_graph(Problem& P, const double* x0_dev, const spock_settings& s
   if (cta) {  // the whole solve in one block (cta.cu): one launch
     const BInst<S> hb = make_binst<S>(P, ws, alpha);
     if (!ws->cta_bi) ws->cta_bi = ws->alloc(sizeof(BInst<S>));
+    // (a copy from pageable memory returns once its source has been read)
     CUDA_TRY(cudaMemcpyAsync(ws->cta_bi, &hb, sizeof(hb), cudaMemcpyHostToDevice, st));
-    CUDA_TRY(cudaStreamSynchronize(st));  // hb lives on this stack frame
     CUDA_TRY(cudaEventRecord(ws->e0, st));
     launch_solve_cta<S>((const BInst<S>*)ws->cta_bi, 1, P.nx + P.nu, mem, max_rounds, trace_dev, st);
     check_launch();
@@ -788,12 +806,13 @@ static int solve_graph(Problem& P, const double* x0_dev, const spock_settings& s
   convert<double, S>(TV, z_dev, nz, st);
   convert<double, S>(TV + nz, eta_dev, P.off.n_eta, st);
   check_launch();
-  SmState fin;
-  CUDA_TRY(cudaMemcpyAsync(&fin, ws->st, sizeof(SmState), cudaMemcpyDeviceToHost, st));
+  CUDA_TRY(cudaMemcpyAsync(ws->h_state, ws->st, sizeof(SmState), cudaMemcpyDeviceToHost, st));
+  CUDA_TRY(cudaMemcpyAsync(ws->h_done + 2, P.err, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
   if (trace_dev)
     CUDA_TRY(cudaMemcpyAsync(s.trace, trace_dev, sizeof(int32_t) * 2 * (size_t)max_iter, cudaMemcpyDeviceToHost,
                              st));
   CUDA_TRY(cudaStreamSynchronize(st));
+  const SmState& fin = *ws->h_state;
   float ms = 0.f;
   cudaEventElapsedTime(&ms, ws->e0, ws->e1);
   const int final_action = fin.done ? fin.action : A_MAXIT;
@@ -824,7 +843,7 @@ static int solve_graph(Problem& P, const double* x0_dev, const spock_settings& s
     for (int g = 0; g < Profiler::kGroups; ++g) info->t_group_ms[g] = ws->prof.on ? ws->prof.acc[g] : 0.0;
   }
   ws->prof.on = false;
-  check_device_flag(P, st);
+  check_device_flag(P, st, ws->h_done + 2);
   if (status == SPOCK_ERR_NUMERICAL) return fail(status, "non-finite residual during the iteration");
   return status;
 }
@@ -868,18 +887,13 @@ static int cp_impl(Problem& P, const double* x0_dev, int k, double alpha, double
   convert<double, S>(a, z_dev, nz, st);
   convert<double, S>(a + nz, eta_dev, P.off.n_eta, st);
   check_launch();
-  if (xi_out) {
-    if (k > 0) {
-      double h[8];
-      CUDA_TRY(cudaMemcpyAsync(h, ws->stats, sizeof(h), cudaMemcpyDeviceToHost, st));
-      CUDA_TRY(cudaStreamSynchronize(st));
-      *xi_out = std::max(h[ST_XIP], h[ST_XID]);
-    } else {
-      *xi_out = NAN;
-    }
-  }
+  double* h = ws->h_state->stats_cur;
+  if (xi_out && k > 0)
+    CUDA_TRY(cudaMemcpyAsync(h, ws->stats, sizeof(double) * 8, cudaMemcpyDeviceToHost, st));
+  CUDA_TRY(cudaMemcpyAsync(ws->h_done + 2, P.err, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
   CUDA_TRY(cudaStreamSynchronize(st));
-  check_device_flag(P, st);
+  check_device_flag(P, st, ws->h_done + 2);
+  if (xi_out) *xi_out = k > 0 ? std::max(h[ST_XIP], h[ST_XID]) : NAN;
   return SPOCK_OK;
 }
 
@@ -927,6 +941,7 @@ struct Batch {
   size_t tab_bytes = 0;
   SmState* st_stage = nullptr;   // staging of the instances' states
   int st_stage_n = 0;
+  cudaEvent_t e0 = nullptr, e1 = nullptr;   // the batch solve's time
   std::vector<int32_t*> bufs;
   void free_plan() {
     if (gexec) cudaGraphExecDestroy(gexec);
@@ -950,6 +965,8 @@ struct Batch {
     if (tab_dev) cudaFree(tab_dev);
     if (tab_host) cudaFreeHost(tab_host);
     if (st_stage) cudaFree(st_stage);
+    if (e0) cudaEventDestroy(e0);
+    if (e1) cudaEventDestroy(e1);
   }
   // uploads one block map from per-instance block counts (and stages)
   DevMap make_map(const std::vector<int>& cnt, const std::vector<int>& stage) {
@@ -978,6 +995,12 @@ struct Batch {
   }
 };
 
+// Error flags of the instances' problems (one copy for the batch).
+template <typename S>
+__global__ void k_gather_err(const BInst<S>* __restrict__ bi, int n, int32_t* __restrict__ out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) out[i] = *bi[i].kp.err;
+}
 __global__ void k_gather_done(SmState* const* __restrict__ sts, int n, int32_t* __restrict__ out) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) out[i] = sts[i]->done;
@@ -1388,9 +1411,9 @@ static int batch_solve(Batch& B, const double* const* x0, const spock_settings& 
     CUDA_TRY(cudaMemcpy(B.st_ptrs, h.data(), sizeof(SmState*) * n, cudaMemcpyHostToDevice));
   }
   int64_t rounds = 0, graph_launches = 0;
-  cudaEvent_t e0, e1;
-  CUDA_TRY(cudaEventCreate(&e0));
-  CUDA_TRY(cudaEventCreate(&e1));
+  if (!B.e0) CUDA_TRY(cudaEventCreate(&B.e0));
+  if (!B.e1) CUDA_TRY(cudaEventCreate(&B.e1));
+  const cudaEvent_t e0 = B.e0, e1 = B.e1;
   CUDA_TRY(cudaEventRecord(e0, B.main));
   if (cfg.cta) {  // one persistent launch: every instance solved by its own block
     launch_solve_cta<S>(bi, n, batch_max_nxu(B), mem, max_rounds, nullptr, B.main);
@@ -1412,8 +1435,6 @@ static int batch_solve(Batch& B, const double* const* x0, const spock_settings& 
   CUDA_TRY(cudaStreamSynchronize(B.main));
   float ms = 0.f;
   cudaEventElapsedTime(&ms, e0, e1);
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
   const int64_t total_launches = cfg.cta ? 1 : B.launches_per_eval + graph_launches * B.g_launches;
   int status = SPOCK_OK;
   std::vector<SmState> fin(n);
@@ -1432,7 +1453,9 @@ static int batch_solve(Batch& B, const double* const* x0, const spock_settings& 
       len.push_back(P.off.n_eta);
     }
     copy_many<S, double>(B, src, dst, len, B.main);
-    batch_states(B, wss, fin.data(), false, B.main);
+    k_gather_err<S><<<(n + 127) / 128, 128, 0, B.main>>>(bi, n, B.done_dev);
+    CUDA_TRY(cudaMemcpyAsync(B.done_host, B.done_dev, sizeof(int32_t) * n, cudaMemcpyDeviceToHost, B.main));
+    batch_states(B, wss, fin.data(), false, B.main);   // synchronises
   }
   for (int i = 0; i < n; ++i) {
     const SmState& f = fin[i];
@@ -1460,7 +1483,7 @@ static int batch_solve(Batch& B, const double* const* x0, const spock_settings& 
       I.fp64_iterations = sizeof(S) == 8 ? f.k : 0;
       I.xi_fp32 = sizeof(S) == 8 ? NAN : f.xi;
     }
-    check_device_flag(*B.probs[i], B.main);
+    check_device_flag(*B.probs[i], B.main, B.done_host + i);
   }
   if (status == SPOCK_ERR_NUMERICAL) return fail(status, "non-finite residual in a batch instance");
   return status;
@@ -2074,6 +2097,10 @@ static int problem_create(const Tree& tree, int32_t nx, int32_t nu, const double
       if (k < nl) par[7][k] = a[u];
       par[8][k] = t.prob[k];
     }
+    if (!gi) {   // the root's box, which every call's x0 is checked against
+      P->root_lo.assign(par[3].begin(), par[3].begin() + nx);
+      P->root_hi.assign(par[4].begin(), par[4].begin() + nx);
+    }
     // ||L||^2 as the largest block norm (remark after the definition of L)
     double best = std::max(0.5, std::max(gh.normL2_xu, gh.normL2_ys));
     for (int32_t k = 0; k < nl && !gi; ++k) {
@@ -2409,9 +2436,7 @@ static int root_box_ok(const Problem& P, const double* x0, cudaStream_t st, bool
       if (!std::isfinite(h[r])) return fail(SPOCK_ERR_NUMERICAL, "x0 is not finite");
     return SPOCK_OK;
   }
-  std::vector<double> lo(P.nx), hi(P.nx);
-  CUDA_TRY(cudaMemcpy(lo.data(), P.f64.xlo, sizeof(double) * P.nx, cudaMemcpyDeviceToHost));
-  CUDA_TRY(cudaMemcpy(hi.data(), P.f64.xhi, sizeof(double) * P.nx, cudaMemcpyDeviceToHost));
+  const std::vector<double>&lo = P.root_lo, &hi = P.root_hi;
   for (int r = 0; r < P.nx; ++r) {
     if (!std::isfinite(h[r])) return fail(SPOCK_ERR_NUMERICAL, "x0 is not finite");
     if (h[r] < lo[r] || h[r] > hi[r]) return fail(SPOCK_ERR_INVALID_ARG, "x0 violates the box of the root node");
@@ -2560,7 +2585,6 @@ int spock_prox_f_dev(spock_problem* p, const double* x0_dev, double alpha, const
     launch_prep<double>(kp, z, (const double*)ws->zero_eta, z_out, sm_count() * 16, st);
     launch_riccati<double>(kp, P->tree.stage_begin, z_out, st, nullptr);
     check_launch();
-    CUDA_TRY(cudaStreamSynchronize(st));
     check_device_flag(*P, st);
     return SPOCK_OK;
   });
@@ -2595,7 +2619,6 @@ int spock_T_dev(spock_problem* p, const double* x0_dev, double alpha, const doub
     launch_dual<double>(kp, DM_DUAL_, false, z, z_out, eta, eta_out, nullptr, nullptr,
                         std::min((P->tree.n + 3) / 4, sm_count() * 16), st);
     check_launch();
-    CUDA_TRY(cudaStreamSynchronize(st));
     check_device_flag(*P, st);
     return SPOCK_OK;
   });
@@ -2790,6 +2813,8 @@ int spock_problem_clone(const spock_problem* base, spock_problem** out) {
       C->nx = B->nx;
       C->nu = B->nu;
       C->normL = B->normL;
+      C->root_lo = B->root_lo;
+      C->root_hi = B->root_hi;
       C->general = B->general;
       C->gd = B->gd;
       C->idx = B->idx;      // read-only index arrays, shared
@@ -2916,7 +2941,6 @@ extern "C" int spock_prox_f_noalloc_dev(spock_problem* p, const double* x0_dev, 
     launch_prep<double>(kp, z, zero_eta, z_out, sm_count() * 16, st);
     launch_riccati<double>(kp, P->tree.stage_begin, z_out, st, nullptr);
     check_launch();
-    CUDA_TRY(cudaStreamSynchronize(st));
     check_device_flag(*P, st);
     return SPOCK_OK;
   });

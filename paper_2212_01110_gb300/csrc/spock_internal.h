@@ -127,6 +127,7 @@ struct Problem {
   bool general = false;   // general form: the L kernels are the matrix-row ones
   GenDims gd;
   double normL = 0.0;
+  std::vector<double> root_lo, root_hi;   // [nx] box of x^0 (box form)
   double factor_seconds = 0.0;
   DevIndex idx;
   int32_t* err = nullptr;  // device flag set by a kernel whose bounded wait gave up
