@@ -30,43 +30,50 @@ namespace spock {
 
 // y[v][j] += sum_q M(e - r0, q) x[v][c0 + q] for the entries e = lane + 32 j
 // in [r0, r0 + nrows), v < NV; M (nrows x ncols) column-major with leading
-// dimension ld.  All lanes of the warp call it (the shuffles).  The next
-// column's entries are loaded while the current column is applied (one
-// column of lookahead: two loads per lane slot in flight).
+// dimension ld.  All lanes of the warp call it (the shuffles).  The entries of
+// U columns are loaded before they are applied: with few nodes per warp the
+// loop is bound by the latency of its loads, and one column of lookahead paid
+// 0.3 us for each of the 700 columns of a node (853 nodes, nx = 50, nu = 20,
+// nc = 80, FP64: L* with the preparation 230 us).  Lane slots without a row
+// are left out: an FP64 multiply-add costs 64 cycles whatever its lanes do.
 template <typename S, int J, int NV, int NA>
 __device__ __forceinline__ void wmv(const S* __restrict__ M, int ld, int nrows, int r0, int ncols, int c0,
                                     const S (&x)[NA][J], S (&y)[NA][J], int lane) {
-  if (ncols <= 0) return;
-  bool live[J];
+  constexpr int U = NV == 1 ? 8 : 4;
+  bool live[J], slot[J];
 #pragma unroll
   for (int j = 0; j < J; ++j) {
     const int r = lane + 32 * j - r0;
     live[j] = r >= 0 && r < nrows;
+    slot[j] = 32 * j < r0 + nrows && 32 * j + 32 > r0;   // warp-uniform
   }
-  auto load = [&](int q, S (&m)[J]) {
-    const S* col = M + (int64_t)q * ld - r0;
 #pragma unroll
-    for (int j = 0; j < J; ++j) m[j] = live[j] ? __ldg(col + lane + 32 * j) : S(0);
-  };
-  S cur[J], nxt[J];
-  load(0, cur);
-  for (int q = 0; q < ncols; ++q) {   // warp-uniform bounds
-    if (q + 1 < ncols) load(q + 1, nxt);
-    const int cq = c0 + q;
-    S xv[NV];
+  for (int js = 0; js < J; ++js) {   // the columns whose vector entries lie in slot js
+    const int qe = min(ncols, 32 * js + 32 - c0);
+    for (int q0 = max(0, 32 * js - c0); q0 < qe; q0 += U) {   // warp-uniform bounds
+      S m[U][J];
 #pragma unroll
-    for (int js = 0; js < J; ++js) {
-      if (js == (cq >> 5)) {
+      for (int i = 0; i < U; ++i) {
+        const S* col = M + (int64_t)(q0 + i) * ld - r0;
 #pragma unroll
-        for (int v = 0; v < NV; ++v) xv[v] = __shfl_sync(kFull, x[v][js], cq & 31);
+        for (int j = 0; j < J; ++j) m[i][j] = live[j] && q0 + i < qe ? __ldg(col + lane + 32 * j) : S(0);
+      }
+#pragma unroll
+      for (int i = 0; i < U; ++i) {
+        if (q0 + i < qe) {
+          S xv[NV];
+#pragma unroll
+          for (int v = 0; v < NV; ++v) xv[v] = __shfl_sync(kFull, x[v][js], (c0 + q0 + i) & 31);
+#pragma unroll
+          for (int j = 0; j < J; ++j) {
+            if (slot[j]) {
+#pragma unroll
+              for (int v = 0; v < NV; ++v) y[v][j] = fma(m[i][j], xv[v], y[v][j]);
+            }
+          }
+        }
       }
     }
-#pragma unroll
-    for (int j = 0; j < J; ++j)
-#pragma unroll
-      for (int v = 0; v < NV; ++v) y[v][j] = fma(cur[j], xv[v], y[v][j]);
-#pragma unroll
-    for (int j = 0; j < J; ++j) cur[j] = nxt[j];
   }
 }
 
