@@ -1261,8 +1261,8 @@ static void batch_init(Batch& B, const std::vector<Workspace*>& wss, const std::
 // single-block persistent solve (cta.cu).  Each candidate runs the
 // evaluation of T at the starting points and kTuneRounds rounds from the
 // same state; the fastest is cached per batch and precision.
-// SPOCK_BATCH_TILE fixes the tile, SPOCK_RICCATI_KERNELS = direct / tma the
-// family, SPOCK_BATCH_MODE = list / cta the mode.
+// SPOCK_BATCH_TILE fixes the tile, SPOCK_RICCATI_KERNELS the family (direct,
+// any other value: staged), SPOCK_BATCH_MODE = list / cta the mode.
 constexpr int kTuneRounds = 4;
 struct BatchCfg {
   int tile, fam;
@@ -1393,7 +1393,7 @@ static int batch_solve(Batch& B, const double* const* x0, const spock_settings& 
     for (int r = 0; r < kBatchRounds; ++r) {
       launch_round_decide_b<S>(bi, n, B.main);
       launch_round_commit_b<S>(bi, B.vec.view(n), B.vec.nblocks, mem, B.main);
-        launch_round_point_b<S>(bi, B.vec.view(n), B.vec.nblocks, mem, B.main);
+      launch_round_point_b<S>(bi, B.vec.view(n), B.vec.nblocks, mem, B.main);
       batch_eval<S>(B, B.main);
     }
     k_gather_done<<<(n + 127) / 128, 128, 0, B.main>>>(B.st_ptrs, n, B.done_dev);
