@@ -247,7 +247,9 @@ __global__ void k_next_basis(int64_t n, const double* __restrict__ u, const doub
 }
 
 __global__ void k_inc(int* kdev) {
-  pdl_enter(); *kdev += 1; }
+  pdl_enter();
+  *kdev += 1;
+}
 
 // red[0] = max |b - u|, red[1] = max |x| (bit patterns of non-negative
 // doubles), r = b - u written out; b = (g, 0)

@@ -512,24 +512,24 @@ __global__ void __launch_bounds__(kMaxSeqThreads + 32, 1) k_fwd_seq_b(const BIns
 // ---------------------------------------------------------------------------
 // launch shapes
 // ---------------------------------------------------------------------------
-static size_t max_dyn_smem() {
-  static size_t v = 0;
-  if (!v) {
-    int dev = 0, b = 0;
+// An attribute of the current device, read once (any thread may be first).
+static int device_attr(cudaDeviceAttr attr, std::atomic<int>& cached) {
+  int v = cached.load(std::memory_order_relaxed);
+  if (v == 0) {
+    int dev = 0;
     cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&b, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    v = (size_t)b;
+    cudaDeviceGetAttribute(&v, attr, dev);
+    cached.store(v, std::memory_order_relaxed);
   }
   return v;
 }
+static size_t max_dyn_smem() {
+  static std::atomic<int> v{0};
+  return (size_t)device_attr(cudaDevAttrMaxSharedMemoryPerBlockOptin, v);
+}
 static int num_sms() {
-  static int v = 0;
-  if (!v) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
-  }
-  return v;
+  static std::atomic<int> v{0};
+  return device_attr(cudaDevAttrMultiProcessorCount, v);
 }
 
 // Threads per block (without the fetching warp): a multiple of 32 that covers
