@@ -68,11 +68,13 @@ void launch_seq_b(int which, const BInst<S>* bi, const BMap& m, int nblocks, con
                   cudaStream_t st);
 // cta.cu: whole solves, one 128-thread block per instance (instances with
 // nx + nu <= max_nxu <= 62, Anderson memory 0, 3 or 5), at most max_rounds
-// rounds each; trace (or NULL) for a single instance.
+// rounds each; bi in device memory.  launch_solve_cta_one: a single instance,
+// handed over by value; trace (or NULL) records its branches.
 bool cta_supported(int nx, int nu, int mem);
 template <typename S>
-void launch_solve_cta(const BInst<S>* bi, int n_inst, int max_nxu, int mem, int64_t max_rounds, int32_t* trace,
-                      cudaStream_t st);
+void launch_solve_cta(const BInst<S>* bi, int n_inst, int max_nxu, int mem, int64_t max_rounds, cudaStream_t st);
+template <typename S>
+void launch_solve_cta_one(const BInst<S>& b, int mem, int64_t max_rounds, int32_t* trace, cudaStream_t st);
 // rounds.cu: the three kernels of a round.
 template <typename S>
 void launch_round_decide_b(const BInst<S>* bi, int n_inst, cudaStream_t st);

@@ -52,11 +52,14 @@ __device__ __forceinline__ void cta_eval(const KP<S>& p, const BInst<S>& b) {
 
 // Block i solves instance i: T of the starting point, then rounds until the
 // state says done or max_rounds rounds have run.  `trace` (or NULL) records
-// the SuperMann branches of a single-instance solve.
+// the SuperMann branches of a single-instance solve.  A batch's instances are
+// read from device memory (bi); a single instance (bi NULL) travels in the
+// launch itself, so that no host object has to outlive a copy of it.
 template <typename S, int J, int SL, int MEM>
-__global__ void __launch_bounds__(128) k_solve_cta(const BInst<S>* __restrict__ bi, int64_t max_rounds,
+__global__ void __launch_bounds__(128) k_solve_cta(const BInst<S>* __restrict__ bi,
+                                                   const __grid_constant__ BInst<S> one, int64_t max_rounds,
                                                    int32_t* trace) {
-  const BInst<S>& b = bi[blockIdx.x];
+  const BInst<S>& b = bi ? bi[blockIdx.x] : one;
   const KP<S> p = b.kp;
   SmState* st = b.st;
   cta_eval<S, J, SL>(p, b);
@@ -83,12 +86,12 @@ bool cta_supported(int nx, int nu, int mem) {
 }
 
 template <typename S>
-void launch_solve_cta(const BInst<S>* bi, int n_inst, int max_nxu, int mem, int64_t max_rounds, int32_t* trace,
-                      cudaStream_t st) {
+static void launch_cta(const BInst<S>* bi, const BInst<S>& one, int n_inst, int max_nxu, int mem, int64_t max_rounds,
+                       int32_t* trace, cudaStream_t st) {
   const bool small = max_nxu <= 30;
 #define SPOCK_CTA(M)                                                                              \
-  if (small) k_solve_cta<S, 1, 1, M><<<n_inst, 128, 0, st>>>(bi, max_rounds, trace);            \
-  else k_solve_cta<S, 2, 2, M><<<n_inst, 128, 0, st>>>(bi, max_rounds, trace);
+  if (small) k_solve_cta<S, 1, 1, M><<<n_inst, 128, 0, st>>>(bi, one, max_rounds, trace);       \
+  else k_solve_cta<S, 2, 2, M><<<n_inst, 128, 0, st>>>(bi, one, max_rounds, trace);
   if (mem == 0) {
     SPOCK_CTA(0)
   } else if (mem == 3) {
@@ -99,7 +102,19 @@ void launch_solve_cta(const BInst<S>* bi, int n_inst, int max_nxu, int mem, int6
 #undef SPOCK_CTA
 }
 
-template void launch_solve_cta<double>(const BInst<double>*, int, int, int, int64_t, int32_t*, cudaStream_t);
-template void launch_solve_cta<float>(const BInst<float>*, int, int, int, int64_t, int32_t*, cudaStream_t);
+template <typename S>
+void launch_solve_cta(const BInst<S>* bi, int n_inst, int max_nxu, int mem, int64_t max_rounds, cudaStream_t st) {
+  launch_cta<S>(bi, BInst<S>{}, n_inst, max_nxu, mem, max_rounds, nullptr, st);
+}
+template <typename S>
+void launch_solve_cta_one(const BInst<S>& b, int mem, int64_t max_rounds, int32_t* trace, cudaStream_t st) {
+  launch_cta<S>(nullptr, b, 1, b.kp.nx + b.kp.nu, mem, max_rounds, trace, st);
+}
+
+#define SPOCK_CTA_INST(S)                                                                          \
+  template void launch_solve_cta<S>(const BInst<S>*, int, int, int, int64_t, cudaStream_t);        \
+  template void launch_solve_cta_one<S>(const BInst<S>&, int, int64_t, int32_t*, cudaStream_t);
+SPOCK_CTA_INST(double)
+SPOCK_CTA_INST(float)
 
 }  // namespace spock

@@ -177,7 +177,6 @@ struct Workspace {
   int g_trace = -1, g_launches_per_round = 0;
   int32_t* h_done = nullptr;  // pinned: done and rounds, [2] the problem's error flag
   SmState* h_state = nullptr; // pinned: the state at the end of a solve; its statistics also for CP steps
-  void* cta_bi = nullptr;      // instance view of the single-block solve (device)
   std::vector<void*> allocs;
   ~Workspace() {
     if (gexec) cudaGraphExecDestroy(gexec);
@@ -748,12 +747,8 @@ static int solve_graph(Problem& P, const double* x0_dev, const spock_settings& s
   ws->launches = 0;
   const int64_t max_rounds = (int64_t)(max_iter + 1) * (h.max_back + 3) + 2;
   if (cta) {  // the whole solve in one block (cta.cu): one launch
-    const BInst<S> hb = make_binst<S>(P, ws, alpha);
-    if (!ws->cta_bi) ws->cta_bi = ws->alloc(sizeof(BInst<S>));
-    // (a copy from pageable memory returns once its source has been read)
-    CUDA_TRY(cudaMemcpyAsync(ws->cta_bi, &hb, sizeof(hb), cudaMemcpyHostToDevice, st));
     CUDA_TRY(cudaEventRecord(ws->e0, st));
-    launch_solve_cta<S>((const BInst<S>*)ws->cta_bi, 1, P.nx + P.nu, mem, max_rounds, trace_dev, st);
+    launch_solve_cta_one<S>(make_binst<S>(P, ws, alpha), mem, max_rounds, trace_dev, st);
     check_launch();
     ws->launches = 1;
   } else {
@@ -1344,8 +1339,8 @@ static BatchCfg batch_tune(Batch& B, const std::vector<Workspace*>& wss, const s
     batch_plan<S>(B, wss, alphas, mem, pick.tile, pick.fam);
     const int n = (int)B.probs.size(), nxu = batch_max_nxu(B);
     const BInst<S>* bi = (const BInst<S>*)B.bi_dev;
-    timed([&] { launch_solve_cta<S>(bi, n, nxu, mem, 1, nullptr, B.main); });  // warm-up
-    const float ms = timed([&] { launch_solve_cta<S>(bi, n, nxu, mem, kTuneRounds, nullptr, B.main); });
+    timed([&] { launch_solve_cta<S>(bi, n, nxu, mem, 1, B.main); });  // warm-up
+    const float ms = timed([&] { launch_solve_cta<S>(bi, n, nxu, mem, kTuneRounds, B.main); });
     if (ms < best) {
       best = ms;
       pick.cta = true;
@@ -1416,7 +1411,7 @@ static int batch_solve(Batch& B, const double* const* x0, const spock_settings& 
   const cudaEvent_t e0 = B.e0, e1 = B.e1;
   CUDA_TRY(cudaEventRecord(e0, B.main));
   if (cfg.cta) {  // one persistent launch: every instance solved by its own block
-    launch_solve_cta<S>(bi, n, batch_max_nxu(B), mem, max_rounds, nullptr, B.main);
+    launch_solve_cta<S>(bi, n, batch_max_nxu(B), mem, max_rounds, B.main);
     check_launch();
   } else {
     batch_eval<S>(B, B.main);  // T of the starting points
