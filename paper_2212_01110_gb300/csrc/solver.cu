@@ -1536,7 +1536,7 @@ static int grad_impl(Problem& P, const double* z, const double* eta, double* gx0
   if (gQN) CUDA_TRY(cudaMemsetAsync(gQN, 0, sizeof(double) * n * nx, st));
   launch_gradient<S>(kp, P.tree.stage_begin, zs, es, w, f.q, gx0, gA, gB, gQ, gR, gQN, maxb, st);
   check_launch();
-  CUDA_TRY(cudaStreamSynchronize(st));
+  check_device_flag(P, st);   // the multipliers' recursion waits for bulk copies; synchronises
   return SPOCK_OK;
 }
 
@@ -1658,7 +1658,10 @@ static int adjoint_impl(Problem& P, const double* z, const double* eta, const do
     CUDA_TRY(cudaStreamSynchronize(st));
     std::memcpy(&rinf, &h[0], sizeof(double));
     std::memcpy(&winf, &h[1], sizeof(double));
-    if (!std::isfinite(rinf)) throw SpockError(SPOCK_ERR_NUMERICAL, "the adjoint solve diverged");
+    if (!std::isfinite(rinf)) {
+      check_device_flag(P, st);   // a wait that gave up is the cause to report
+      throw SpockError(SPOCK_ERR_NUMERICAL, "the adjoint solve diverged");
+    }
   };
   int it = 0;   // applications of J^T inside the Arnoldi steps
   std::vector<double> H((size_t)(m + 1) * m), cs(m), sn(m), gam(m + 1), hv, y(m);
@@ -2663,6 +2666,19 @@ int spock_grad(spock_problem* p, const double* z, const double* eta, int32_t pre
         {g_Q, gQ, n * nx}, {g_R, gR, n * nu}, {g_QN, gQN, n * nx}};
     for (const auto& o : outs)
       if (o.host) CUDA_TRY(cudaMemcpy(o.host, o.dev, sizeof(double) * o.len, cudaMemcpyDeviceToHost));
+    return SPOCK_OK;
+  });
+}
+
+// For the tests (not in spock.h): the state a kernel whose bounded wait gave up
+// leaves behind.  The next call that launches such kernels reports it.
+int spock_internal_raise_wait_flag(spock_problem* p) {
+  return guarded([&]() -> int {
+    Problem* P = as_problem(p);
+    if (!P) return fail(SPOCK_ERR_INVALID_ARG, "NULL argument");
+    CUDA_TRY(cudaSetDevice(P->device));
+    const int32_t one = 1;
+    CUDA_TRY(cudaMemcpy(P->err, &one, sizeof(one), cudaMemcpyHostToDevice));
     return SPOCK_OK;
   });
 }
