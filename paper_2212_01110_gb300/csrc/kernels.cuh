@@ -11,8 +11,6 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
-#include "fxp.cuh"
-
 namespace spock {
 
 // bytes, rounded up to a multiple of 16 or 128
@@ -121,16 +119,14 @@ struct KP {
   const S* __restrict__ NB;
   const S* __restrict__ Kt;
   // the factors as the sequence kernels read them (riccati_seq.cu), per matrix
-  // one 16-byte aligned block of gbB, gfB, nbB, ktB bytes, row-major:
+  // one 128-byte aligned block of gbB, gfB, nbB, ktB bytes, row-major:
   //   pGb  [B | Abar] (nx x (nu + nx)),  pGf  [Abar | B]^T ((nx + nu) x nx),
   //   pNB  [Rtilde^-1 | E] (nu x (nu + nx)) and K (nu x nx), E = Rtilde^-1 (K + W^T),
   //   pKt  K^T (nx x nu).
-  // FP32: numbers.  FP64: fixed-point entries (fxp.cuh) followed by one exponent
-  // per column (pNB: per column of the first matrix, E's also for K's).
-  const unsigned char* __restrict__ pGb;
-  const unsigned char* __restrict__ pGf;
-  const unsigned char* __restrict__ pNB;
-  const unsigned char* __restrict__ pKt;
+  const S* __restrict__ pGb;
+  const S* __restrict__ pGf;
+  const S* __restrict__ pNB;
+  const S* __restrict__ pKt;
   uint32_t gbB, gfB, nbB, ktB;
   S* __restrict__ hb;   // [n - 1][hst] [B^c | Abar^c]^T q^c of the nonroot nodes
   int32_t hst;

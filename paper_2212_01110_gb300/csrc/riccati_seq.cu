@@ -25,18 +25,20 @@
 // of D slots (address arithmetic, fence and copies in one of the T threads
 // would lengthen every step, and so would a second barrier to wait on: 200
 // cycles each, measured).  What latency is left, and the serial sums and
-// barriers of a step, is covered by the other blocks of the SM.  FP64 products
-// are the exact integer sums of fxp.cuh.
+// barriers of a step, is covered by the other blocks of the SM.
+//
+// FP64 factors and vectors are held and multiplied as doubles.  (A form with
+// 57-bit integers relative to a column's largest entry and exact integer sums
+// ran the chains below in 670 and 473 us, but entries far below the largest
+// lost digits without limit: a dynamics residual of 1e-10 for states whose units
+// differ by 1e6, 5e-4 by 1e12, against 2e-15.)
 //
 // What bounds it and what it measured (GB300, nx = 50, nu = 20).  Chains of the
-// 62,805-node tree, FP64: backward 670 us (2.84 GB, 4.2 TB/s), forward 473 us
-// (2.2 GB), where direct-load kernels on the FP64 pipe took 1,073 and 705 us;
-// the FP32 chains of 4,096 sequences of five nodes run at 5.2 - 5.6 TB/s.  A
-// step alone takes 3.5 (backward) and 2.1 us (forward) in FP64, against 15.9
-// and 4.3, and 1.3 and 0.9 us in FP32, against 2.7 and 1.8.  The FP64 chains
-// are bound by the steps of the four resident blocks (about 28 cycles a row of
-// five wide multiply-adds and two shared loads, and 1,000 instructions of
-// conversions and barriers), the FP32 ones by memory latency.
+// 62,805-node tree, FP64: backward 837 us (2.75 GB), forward 611 us (2.2 GB),
+// where direct-load kernels took 1,073 and 705 us; the FP32 chains of 4,096
+// sequences of five nodes run at 5.2 - 5.6 TB/s.  The FP64 chains are bound by
+// the FP64 pipes (1.9 multiply-adds per clock and SM: a warp instruction holds
+// its sub-partition's pipe for 64 cycles), the FP32 ones by memory latency.
 //
 // Bounded waits: a wait that exceeds kWaitLimit polls sets *p.err and the
 // thread stops waiting (the fetching warp: stops issuing); the block finishes
@@ -54,9 +56,9 @@
 
 namespace spock {
 
-constexpr int kMaxSeqThreads = 256;   // T; 32 more fetch
-constexpr int kMaxSlots = 8;
-
+constexpr int kMaxSeqThreads = 224;   // T; 32 more fetch
+constexpr int kMaxSlots = 2;
+constexpr int kMaxGroups = 4;         // row groups of an FP64 product
 
 // Shared memory of a block, in bytes: D slots of one node's blocks each,
 // prepared vectors, partial sums.
@@ -68,52 +70,69 @@ __host__ __device__ inline int up4(int n) { return (n + 3) & ~3; }
 template <typename S>
 __host__ __device__ inline SeqLayout seq_layout_bwd(const KP<S>& p, int T) {
   SeqLayout L;
-  const uint32_t V = sizeof(typename Fx<S>::Vec);
   L.item = up128(p.gbB + p.nbB + (p.xs + p.us) * (uint32_t)sizeof(S));   // [B | Abar] | node block | xbar | ubar
-  L.vecA = up16(2 * up4(p.nu) * V);                               // (g; -ubar)
-  L.vecB = up16(up4(p.nx) * V);                                   // q
-  L.part = up16(T * (uint32_t)sizeof(typename Fx<S>::Acc));
+  L.vecA = up16(2 * up4(p.nu) * (uint32_t)sizeof(S));                               // (g; -ubar)
+  L.vecB = up16(up4(p.nx) * (uint32_t)sizeof(S));                                   // q
+  L.part = up16(T * (uint32_t)sizeof(S));
   return L;
 }
 template <typename S>
 __host__ __device__ inline SeqLayout seq_layout_fwd(const KP<S>& p, int T) {
   SeqLayout L;
-  const uint32_t V = sizeof(typename Fx<S>::Vec);
   L.item = up128(p.gfB + p.ktB + p.us * (uint32_t)sizeof(S));   // [Abar | B]^T | K^T of the parent | d of the node
-  L.vecA = up16(up4(p.nx + p.nu) * V);                   // (x; d) of the parent and of the node
+  L.vecA = up16(up4(p.nx + p.nu) * (uint32_t)sizeof(S));                   // (x; d) of the parent and of the node
   L.vecB = L.vecA;
-  L.part = up16(T * (uint32_t)sizeof(typename Fx<S>::Acc));
+  L.part = up16(T * (uint32_t)sizeof(S));
   return L;
 }
 
 // Barrier of the T working threads of a block.
 __device__ __forceinline__ void seq_bar(int T) { named_bar(1, T); }
 
-// Columns of a product: two blocks of n0 and n1, the second one from a warp
-// boundary on (both in one warp when they fit), so that no warp runs the sums
-// of both: with n0 = 50 and n1 = 20 packed into 70 threads, one warp ran 120
-// rows where the others ran 70.
-__host__ __device__ inline int seq_off(int n0, int n1) { return n0 + n1 <= 32 ? n0 : (n0 + 31) & ~31; }
-__host__ __device__ inline int seq_cols(int n0, int n1) { return (seq_off(n0, n1) + n1 + 31) & ~31; }
+// Columns of a product: two blocks of n0 and n1, thread (row group, column).
+// FP32: the second block from a warp boundary on (both in one warp when they
+// fit), so that no warp runs the sums of both: with n0 = 50 and n1 = 20 packed
+// into 70 threads, one warp ran 120 rows where the others ran 70.  FP64: a warp
+// instruction holds its sub-partition's FP64 pipe for 64 cycles whatever its
+// lanes do, so the columns of all row groups are packed and few lanes idle
+// (nx = 50, nu = 20, three groups: 210 of 224 lanes).
+template <typename S>
+__host__ __device__ inline int seq_off(int n0, int n1) {
+  return sizeof(S) == 8 || n0 + n1 <= 32 ? n0 : (n0 + 31) & ~31;
+}
+template <typename S>
+__host__ __device__ inline int seq_cols(int n0, int n1) {
+  return sizeof(S) == 8 ? n0 + n1 : (seq_off<S>(n0, n1) + n1 + 31) & ~31;
+}
+// Row groups of a product of CP columns in T threads, and the rows of each.
+template <typename S>
+__device__ __forceinline__ int seq_groups(int T, int CP) {
+  return sizeof(S) == 8 ? min(T / CP, kMaxGroups) : T / CP;
+}
+template <typename S>
+__device__ __forceinline__ int seq_chunk(int n, int RG) {
+  const int c = (n + RG - 1) / RG;
+  return sizeof(S) == 8 ? c : up4(c);   // FP32 reads the vector in 16-byte pieces
+}
 
-// acc += sum over n rows of M[r] v[r]; `m` the shared-memory address of the
-// thread's entry in the first row, rows ldB bytes apart, `v` that of the
-// prepared vector (16-byte aligned).  Eight rows are loaded before their
-// products, without a branch among them.
-__device__ __forceinline__ void seq_rows(Fx<float>::Acc& acc, uint32_t m, uint32_t ldB, uint32_t v, int n) {
+// acc + sum over n rows of M[r] v[r]; `m` the shared-memory address of the
+// thread's entry in the first row, rows ldB bytes apart, `v` that of the vector
+// (FP32: 16-byte aligned).  FP32: eight rows are loaded before their products,
+// without a branch among them.
+__device__ __forceinline__ float seq_rows(float acc, uint32_t m, uint32_t ldB, uint32_t v, int n) {
   for (; n >= 8; n -= 8, m += 8 * ldB, v += 32) {
     float a[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) a[i] = lds_f32(m + i * ldB);
     const float4 x = lds_f32x4(v), y = lds_f32x4(v + 16);
-    acc.v = fmaf(a[0], x.x, acc.v);
-    acc.v = fmaf(a[1], x.y, acc.v);
-    acc.v = fmaf(a[2], x.z, acc.v);
-    acc.v = fmaf(a[3], x.w, acc.v);
-    acc.v = fmaf(a[4], y.x, acc.v);
-    acc.v = fmaf(a[5], y.y, acc.v);
-    acc.v = fmaf(a[6], y.z, acc.v);
-    acc.v = fmaf(a[7], y.w, acc.v);
+    acc = fmaf(a[0], x.x, acc);
+    acc = fmaf(a[1], x.y, acc);
+    acc = fmaf(a[2], x.z, acc);
+    acc = fmaf(a[3], x.w, acc);
+    acc = fmaf(a[4], y.x, acc);
+    acc = fmaf(a[5], y.y, acc);
+    acc = fmaf(a[6], y.z, acc);
+    acc = fmaf(a[7], y.w, acc);
   }
   if (n > 0) {
     float a[7], x[7];
@@ -125,45 +144,31 @@ __device__ __forceinline__ void seq_rows(Fx<float>::Acc& acc, uint32_t m, uint32
     }
 #pragma unroll
     for (int i = 0; i < 7; ++i)
-      if (i < n) acc.v = fmaf(a[i], x[i], acc.v);
+      if (i < n) acc = fmaf(a[i], x[i], acc);
   }
+  return acc;
 }
-__device__ __forceinline__ void seq_rows(Fx<double>::Acc& acc, uint32_t m, uint32_t ldB, uint32_t v, int n) {
+__device__ __forceinline__ double seq_rows(double acc, uint32_t m, uint32_t ldB, uint32_t v, int n) {
   const char* mp = (const char*)__cvta_shared_to_generic(m);
-  const int4* vp = (const int4*)__cvta_shared_to_generic(v);
+  const double* vp = (const double*)__cvta_shared_to_generic(v);
   __builtin_assume(__isShared(mp));
   __builtin_assume(__isShared(vp));
 #pragma unroll 4
-  for (int r = 0; r < n; ++r, mp += ldB) Fx<double>::mad(acc, *(const int2*)mp, vp[r]);
+  for (int r = 0; r < n; ++r, mp += ldB) acc = fma(*(const double*)mp, vp[r], acc);
+  return acc;
 }
 
-// Sum of the row groups' accumulators in the threads of row group 0 (one
-// barrier if there is more than one group; every thread calls it).
+// Sum of the row groups' accumulators in the threads of row group 0, a column's
+// threads `step` apart (one barrier if there is more than one group; every
+// thread calls it).
 template <typename S>
-__device__ __forceinline__ void seq_reduce(typename Fx<S>::Acc& acc, int rg, int RG, int CP, bool live,
-                                           typename Fx<S>::Acc* part, int T) {
-  if (RG == 1) return;
+__device__ __forceinline__ S seq_reduce(S acc, int rg, int RG, int step, bool live, S* part, int T) {
+  if (RG == 1) return acc;
   if (live && rg > 0) part[threadIdx.x] = acc;
   seq_bar(T);
   if (live && rg == 0)
-    for (int i = 1; i < RG; ++i) Fx<S>::add(acc, part[i * CP + threadIdx.x]);
-}
-
-// Largest key over threads 0 .. n - 1 (key is 0 elsewhere), to those threads;
-// a barrier when they span several warps.  FP32: nothing.
-template <typename S>
-__device__ __forceinline__ uint32_t seq_kmax(uint32_t key, int n, uint32_t* word, int T) {
-  if (sizeof(S) == 4) return 0u;
-  key = __reduce_max_sync(kFull, key);
-  if (n <= 32) return key;   // warp 0 holds all of them
-  const int w = threadIdx.x >> 5;
-  if ((threadIdx.x & 31) == 0 && w < 5) word[w] = key;
-  seq_bar(T);
-  const uint4 k4 = *reinterpret_cast<const uint4*>(word);
-  key = max(k4.x, k4.y);
-  if (n > 64) key = max(key, max(k4.z, k4.w));
-  if (n > 128) key = max(key, word[4]);
-  return key;
+    for (int i = 1; i < RG; ++i) acc += part[i * step + threadIdx.x];
+  return acc;
 }
 
 // The ring: per slot a barrier for "full" (the copies have arrived) and one for
@@ -232,22 +237,15 @@ __device__ __forceinline__ void seq_fetch(SeqRing& ring, const int32_t* skip, co
 template <typename S, bool LAM>
 __device__ __forceinline__ void bwd_seq_body(const KP<S>& p, int t_hi, int t_lo, int bid, int nblk, int D,
                                              S* lam = nullptr) {
-  using Mat = typename Fx<S>::Mat;
-  using Vec = typename Fx<S>::Vec;
-  using Acc = typename Fx<S>::Acc;
-  constexpr bool FX = sizeof(S) == 8;
-  constexpr uint32_t MB = sizeof(Mat), VB = sizeof(Vec);
+  constexpr uint32_t B = sizeof(S);
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ uint64_t bars[2][kMaxSlots];
-  __shared__ __align__(16) uint32_t kword[8];
-  __shared__ uint32_t kgs;
   const int tid = threadIdx.x, T = blockDim.x - 32;
   const int nx = p.nx, nu = p.nu, ncol = nx + nu;
   const SeqLayout Ly = seq_layout_bwd(p, T);
   const int cnt = p.stage_begin[t_lo + 1] - p.stage_begin[t_lo];
   if (bid >= cnt) return;
   SeqRing ring{bars[0], bars[1], 0u, false};
-  if (tid < 8) kword[tid] = 0;
   if (tid == 0) {
     for (int s = 0; s < D; ++s) {
       mbar_init(&ring.full[s], 1);
@@ -266,8 +264,8 @@ __device__ __forceinline__ void bwd_seq_body(const KP<S>& p, int t_hi, int t_lo,
           unsigned char* dst = smem + slot * Ly.item;
           uint64_t* bar = &ring.full[slot];
           mbar_expect_tx(bar, xB + (leaf ? 0u : p.nbB + uB) + (k > 0 ? p.gbB : 0u));
-          if (!leaf) bulk_g2s(dst + p.gbB, p.pNB + (size_t)k * p.nbB, p.nbB, bar);
-          if (k > 0) bulk_g2s(dst, p.pGb + (size_t)(k - 1) * p.gbB, p.gbB, bar);
+          if (!leaf) bulk_g2s(dst + p.gbB, reinterpret_cast<const unsigned char*>(p.pNB) + (size_t)k * p.nbB, p.nbB, bar);
+          if (k > 0) bulk_g2s(dst, reinterpret_cast<const unsigned char*>(p.pGb) + (size_t)(k - 1) * p.gbB, p.gbB, bar);
         },
         [&](int slot, int k, int) {
           unsigned char* dst = smem + slot * Ly.item + p.gbB + p.nbB;
@@ -278,18 +276,19 @@ __device__ __forceinline__ void bwd_seq_body(const KP<S>& p, int t_hi, int t_lo,
   }
   pdl_enter();
   if (p.skip && *p.skip) return;
-  Vec* const A = reinterpret_cast<Vec*>(smem + D * Ly.item);               // (g; -ubar), 4-entry aligned halves
-  Vec* const B = reinterpret_cast<Vec*>(smem + D * Ly.item + Ly.vecA);     // q
-  Acc* const part = reinterpret_cast<Acc*>(smem + D * Ly.item + Ly.vecA + Ly.vecB);
-  const uint32_t aA = smem_u32(A), aB = smem_u32(B), a0 = smem_u32(smem);
+  S* const vA = reinterpret_cast<S*>(smem + D * Ly.item);               // (g; -ubar), 16-byte aligned halves
+  S* const vB = reinterpret_cast<S*>(smem + D * Ly.item + Ly.vecA);     // q
+  S* const part = reinterpret_cast<S*>(smem + D * Ly.item + Ly.vecA + Ly.vecB);
+  const uint32_t aA = smem_u32(vA), aB = smem_u32(vB), a0 = smem_u32(smem);
   // column col of row group rg: d and h_u in columns 0 .. nu - 1, q and h_x from
   // column off on; mc the column in the matrices [.. (nu) | .. (nx)]; row group
   // rg takes rows u0 .. or x0 .. of a vector
-  const int off = seq_off(nu, nx), CP = seq_cols(nu, nx), RG = T / CP, rg = tid / CP, col = tid - rg * CP;
+  const int off = seq_off<S>(nu, nx), CP = seq_cols<S>(nu, nx), RG = seq_groups<S>(T, CP);
+  const int rg = tid / CP, col = tid - rg * CP;
   const bool inu = tid < nu, inx = tid >= off && tid < off + nx, own = inu || inx;
   const bool live = rg < RG && (col < nu || (col >= off && col < off + nx));
   const int mc = col < nu ? col : col - off + nu, ex = tid - off;
-  const int nu4 = up4(nu), cu = up4((nu + RG - 1) / RG), cx = up4((nx + RG - 1) / RG);
+  const int nu4 = up4(nu), cu = seq_chunk<S>(nu, RG), cx = seq_chunk<S>(nx, RG);
   const int u0 = rg * cu, un = max(0, min(cu, nu - u0)), x0 = rg * cx, xn = max(0, min(cx, nx - x0));
   S h = S(0);   // h of the current node: this thread's column
   int slot = 0;
@@ -312,48 +311,41 @@ __device__ __forceinline__ void bwd_seq_body(const KP<S>& p, int t_hi, int t_lo,
       if (leaf) {
         if (inx) q = -xb[ex];
       } else {
-        const S u = inu ? (LAM ? h : (xb + p.xs)[tid]) : S(0);
-        const S g = !LAM && inu ? u - h : S(0);
-        const S base = inx ? h - xb[ex] : S(0);
-        const uint32_t kg = seq_kmax<S>(inu ? max(Fx<S>::key(g), Fx<S>::key(u)) : 0u, nu, kword, T);
         if (inu) {
-          A[tid] = Fx<S>::vec(g, kg);
-          A[nu4 + tid] = Fx<S>::vec(-u, kg);
+          const S u = LAM ? h : (xb + p.xs)[tid];
+          vA[tid] = LAM ? S(0) : u - h;   // g
+          vA[nu4 + tid] = -u;
         }
-        if (FX && tid == 0) kgs = kg;
+        const S base = inx ? h - xb[ex] : S(0);
         seq_bar(T);
-        Acc acc;
-        Fx<S>::zero(acc);
+        S acc = S(0);
         if (live) {   // [Rt^-1 | E] (nu x ncol), then K (nu x nx)
-          const uint32_t m1 = ait + p.gbB, m2 = m1 + nu * ncol * MB;
-          seq_rows(acc, m1 + (u0 * ncol + mc) * MB, ncol * MB, aA + u0 * VB, un);
-          if (col >= off) seq_rows(acc, m2 + (u0 * nx + mc - nu) * MB, nx * MB, aA + (nu4 + u0) * VB, un);
+          const uint32_t m1 = ait + p.gbB, m2 = m1 + nu * ncol * B;
+          acc = seq_rows(acc, m1 + (u0 * ncol + mc) * B, ncol * B, aA + u0 * B, un);
+          if (col >= off) acc = seq_rows(acc, m2 + (u0 * nx + mc - nu) * B, nx * B, aA + (nu4 + u0) * B, un);
         }
-        seq_reduce<S>(acc, rg, RG, CP, live, part, T);
-        if (own) {
-          const int* xn_ = reinterpret_cast<const int*>(it + p.gbB + (nu * ncol + nu * nx) * MB);
-          const S v = Fx<S>::value(acc, FX ? Fx<S>::vec_exp(kgs) + xn_[mc] : 0);
-          if (inx) q = base + v;
-          if (LAM) {
-            if (inx) lam[(int64_t)k * p.xs + ex] = q;
-          } else if (inu) {
-            p.d[(int64_t)k * p.us + tid] = v;
-          }
+        acc = seq_reduce<S>(acc, rg, RG, CP, live, part, T);
+        if (inx) q = base + acc;
+        if (LAM) {
+          if (inx) lam[(int64_t)k * p.xs + ex] = q;
+        } else if (inu) {
+          p.d[(int64_t)k * p.us + tid] = acc;
         }
       }
       if (k > 0) {
-        const uint32_t kq = seq_kmax<S>(inx ? Fx<S>::key(q) : 0u, CP, kword, T);
-        if (inx) B[ex] = Fx<S>::vec(q, kq);
+        if (inx) vB[ex] = q;
         seq_bar(T);
-        Acc acc;
-        Fx<S>::zero(acc);
-        if (live) seq_rows(acc, ait + (x0 * ncol + mc) * MB, ncol * MB, aB + x0 * VB, xn);
-        seq_reduce<S>(acc, rg, RG, CP, live, part, T);
+        S acc = S(0);
+        if (live) acc = seq_rows(acc, ait + (x0 * ncol + mc) * B, ncol * B, aB + x0 * B, xn);
+        acc = seq_reduce<S>(acc, rg, RG, CP, live, part, T);
         if (own) {
-          h = Fx<S>::value(acc, FX ? Fx<S>::vec_exp(kq) + reinterpret_cast<const int*>(it + nx * ncol * MB)[mc] : 0);
+          h = acc;
           if (t == t_lo) p.hb[(int64_t)(k - 1) * p.hst + mc] = h;
         }
-        seq_bar(T);   // every thread is through with the slot and the vectors
+        // every thread is through with the slot and the vectors; with several row
+        // groups the barrier of the sum has said so (what group 0 reads after it,
+        // the others' sums, is written again behind the next node's first barrier)
+        if (RG == 1) seq_bar(T);
         if (tid == 0) mbar_arrive(&ring.empty[slot]);
       }
       if (++slot == D) slot = 0;
@@ -365,21 +357,15 @@ __device__ __forceinline__ void bwd_seq_body(const KP<S>& p, int t_hi, int t_lo,
 template <typename S>
 __device__ __forceinline__ void fwd_seq_body(const KP<S>& p, int t_lo, int t_hi, S* __restrict__ zo, int bid,
                                              int nblk, int D) {
-  using Mat = typename Fx<S>::Mat;
-  using Vec = typename Fx<S>::Vec;
-  using Acc = typename Fx<S>::Acc;
-  constexpr bool FX = sizeof(S) == 8;
-  constexpr uint32_t MB = sizeof(Mat), VB = sizeof(Vec);
+  constexpr uint32_t B = sizeof(S);
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ uint64_t bars[2][kMaxSlots];
-  __shared__ __align__(16) uint32_t kword[2][8];
   const int tid = threadIdx.x, T = blockDim.x - 32;
   const int nx = p.nx, nu = p.nu, ncol = nx + nu;
   const SeqLayout Ly = seq_layout_fwd(p, T);
   const int cnt = p.stage_begin[t_lo + 1] - p.stage_begin[t_lo];
   if (bid >= cnt) return;
   SeqRing ring{bars[0], bars[1], 0u, false};
-  if (tid < 16) kword[tid >> 3][tid & 7] = 0;
   if (tid == 0) {
     for (int s = 0; s < D; ++s) {
       mbar_init(&ring.full[s], 1);
@@ -399,8 +385,8 @@ __device__ __forceinline__ void fwd_seq_body(const KP<S>& p, int t_lo, int t_hi,
           unsigned char* dst = smem + slot * Ly.item;
           uint64_t* bar = &ring.full[slot];
           mbar_expect_tx(bar, p.gfB + (first ? p.ktB : 0u) + (k < p.nl ? uB : 0u));
-          bulk_g2s(dst, p.pGf + (size_t)(k - 1) * p.gfB, p.gfB, bar);
-          if (first) bulk_g2s(dst + p.gfB, p.pKt + (size_t)par * p.ktB, p.ktB, bar);
+          bulk_g2s(dst, reinterpret_cast<const unsigned char*>(p.pGf) + (size_t)(k - 1) * p.gfB, p.gfB, bar);
+          if (first) bulk_g2s(dst + p.gfB, reinterpret_cast<const unsigned char*>(p.pKt) + (size_t)par * p.ktB, p.ktB, bar);
         },
         [&](int slot, int k, int) {
           if (k < p.nl)
@@ -410,19 +396,26 @@ __device__ __forceinline__ void fwd_seq_body(const KP<S>& p, int t_lo, int t_hi,
   }
   pdl_enter();
   if (p.skip && *p.skip) return;
-  Vec* W = reinterpret_cast<Vec*>(smem + D * Ly.item);              // (x; d) of the parent
-  Vec* Y = reinterpret_cast<Vec*>(smem + D * Ly.item + Ly.vecA);    // (x; d) of the node
-  Acc* const part = reinterpret_cast<Acc*>(smem + D * Ly.item + Ly.vecA + Ly.vecB);
+  S* W = reinterpret_cast<S*>(smem + D * Ly.item);              // (x; d) of the parent
+  S* Y = reinterpret_cast<S*>(smem + D * Ly.item + Ly.vecA);    // (x; d) of the node
+  S* const part = reinterpret_cast<S*>(smem + D * Ly.item + Ly.vecA + Ly.vecB);
   const uint32_t a0 = smem_u32(smem);
-  // columns 0 .. nx - 1: x, from column off on: u of the parent; the threads of
-  // row group 0 also hold the entries of (x; d), entry e
-  const int off = seq_off(nx, nu), CP = seq_cols(nx, nu), RG = T / CP, rg = tid / CP, col = tid - rg * CP;
+  // x (columns of ncol rows), then u of the parent (nx rows).  FP32: both in
+  // each row group.  FP64: the x columns of all groups first, so that few warps
+  // run the longer sums for columns of both (a step of the benchmark's tree:
+  // 154 warp instructions instead of 168).  The threads of row group 0 also
+  // hold the entries of (x; d), entry e.
+  const int CP = seq_cols<S>(nx, nu), RG = seq_groups<S>(T, CP);
+  const int off = sizeof(S) == 8 ? RG * nx : seq_off<S>(nx, nu);
+  const bool xcol = sizeof(S) == 8 ? tid < off : tid % CP < nx;
+  const int step = sizeof(S) == 4 ? CP : (xcol ? nx : nu);
+  const int rg = sizeof(S) == 4 ? tid / CP : (xcol ? tid / nx : (tid - off) / nu);
+  const int col = xcol ? tid - rg * step : tid - off - rg * step;   // of x or of u
   const bool inx = tid < nx, inu = tid >= off && tid < off + nu, own = inx || inu;
-  const int a = tid - off, e = inx ? tid : nx + a, ca = col - off;
-  const int cc = up4((ncol + RG - 1) / RG), cx = up4((nx + RG - 1) / RG);
+  const int a = tid - off, e = inx ? tid : nx + a;
+  const int cc = seq_chunk<S>(ncol, RG), cx = seq_chunk<S>(nx, RG);
   const int w0 = rg * cc, wn = max(0, min(cc, ncol - w0)), x0 = rg * cx, xn = max(0, min(cx, nx - x0));
   S w = S(0);   // entry tid of the parent's (x; d)
-  int ew = 0;   // exponent of W
   int slot = 0;
   for (int ci = bid; ci < cnt; ci += nblk) {
     for (int t = t_lo; t <= t_hi; ++t) {
@@ -436,39 +429,32 @@ __device__ __forceinline__ void fwd_seq_body(const KP<S>& p, int t_lo, int t_hi,
           else if (par > 0) w = zo[p.zx[par] + tid];
           else w = p.x0[tid];
           if (par == 0 && first && inx) zo[p.zx[0] + tid] = w;
+          W[e] = w;
         }
-        const uint32_t kw = seq_kmax<S>(own ? Fx<S>::key(w) : 0u, CP, kword[0], T);
-        if (own) W[e] = Fx<S>::vec(w, kw);
-        ew = Fx<S>::vec_exp(kw);
         seq_bar(T);
       }
       const unsigned char* it = smem + slot * Ly.item;
       const uint32_t ait = a0 + slot * Ly.item, aW = smem_u32(W);
       ring.wait(ring.full, slot, p.err);
-      const bool live = rg < RG && (col < nx || (first && ca >= 0 && ca < nu));
-      Acc acc;
-      Fx<S>::zero(acc);
-      if (live) {   // [Abar | B]^T (ncol x nx) and K^T (nx x nu)
-        if (col < nx) seq_rows(acc, ait + (w0 * nx + col) * MB, nx * MB, aW + w0 * VB, wn);
-        else seq_rows(acc, ait + p.gfB + (x0 * nu + ca) * MB, nu * MB, aW + x0 * VB, xn);
+      const bool live = rg < RG && (xcol || (first && col >= 0 && col < nu));
+      S acc = S(0);
+      if (live) {   // [Abar | B]^T (ncol x nx) and K^T (nx x nu), one loop for both: a warp may hold columns of each
+        acc = seq_rows(acc, ait + (xcol ? (w0 * nx + col) * B : p.gfB + (x0 * nu + col) * B), (xcol ? nx : nu) * B,
+                       aW + (xcol ? w0 : x0) * B, xcol ? wn : xn);
       }
-      seq_reduce<S>(acc, rg, RG, CP, live, part, T);
+      acc = seq_reduce<S>(acc, rg, RG, step, live, part, T);
       if (own && live) {
-        const int* ex = reinterpret_cast<const int*>(inx ? it + ncol * nx * MB : it + p.gfB + nx * nu * MB);
-        const S v = Fx<S>::value(acc, FX ? ew + ex[inx ? tid : a] : 0);
         if (inx) {
-          zo[zxk + tid] = v;
-          w = v;
+          zo[zxk + tid] = acc;
+          w = acc;
         } else {
-          zo[zup + a] = w + v;
+          zo[zup + a] = w + acc;
         }
       }
       if (t < t_hi) {   // the node's (x; d) for the next step
         if (inu) w = reinterpret_cast<const S*>(it + p.gfB + p.ktB)[a];
-        const uint32_t ky = seq_kmax<S>(own ? Fx<S>::key(w) : 0u, CP, kword[1], T);
-        if (own) Y[e] = Fx<S>::vec(w, ky);
-        ew = Fx<S>::vec_exp(ky);
-        Vec* y = W;
+        if (own) Y[e] = w;
+        S* y = W;
         W = Y;
         Y = y;
       }
@@ -480,15 +466,15 @@ __device__ __forceinline__ void fwd_seq_body(const KP<S>& p, int t_lo, int t_hi,
 }
 
 template <typename S>
-__global__ void __launch_bounds__(kMaxSeqThreads + 32, 1) k_bwd_seq(KP<S> p, int t_hi, int t_lo, int D) {
+__global__ void __launch_bounds__(kMaxSeqThreads + 32, sizeof(S) == 8 ? 4 : 1) k_bwd_seq(KP<S> p, int t_hi, int t_lo, int D) {
   bwd_seq_body<S, false>(p, t_hi, t_lo, blockIdx.x, gridDim.x, D);
 }
 template <typename S>
-__global__ void __launch_bounds__(kMaxSeqThreads + 32, 1) k_lambda_seq(KP<S> p, int t_hi, int t_lo, S* lam, int D) {
+__global__ void __launch_bounds__(kMaxSeqThreads + 32, sizeof(S) == 8 ? 4 : 1) k_lambda_seq(KP<S> p, int t_hi, int t_lo, S* lam, int D) {
   bwd_seq_body<S, true>(p, t_hi, t_lo, blockIdx.x, gridDim.x, D, lam);
 }
 template <typename S>
-__global__ void __launch_bounds__(kMaxSeqThreads + 32, 1) k_fwd_seq(KP<S> p, int t_lo, int t_hi, S* __restrict__ zo,
+__global__ void __launch_bounds__(kMaxSeqThreads + 32, sizeof(S) == 8 ? 4 : 1) k_fwd_seq(KP<S> p, int t_lo, int t_hi, S* __restrict__ zo,
                                                             int D) {
   fwd_seq_body<S>(p, t_lo, t_hi, zo, blockIdx.x, gridDim.x, D);
 }
@@ -496,13 +482,13 @@ __global__ void __launch_bounds__(kMaxSeqThreads + 32, 1) k_fwd_seq(KP<S> p, int
 // Batched: block -> (instance, block) from the launch's map; stage < 0: the
 // chain region of every instance (forward: below the root at the earliest).
 template <typename S>
-__global__ void __launch_bounds__(kMaxSeqThreads + 32, 1) k_bwd_seq_b(const BInst<S>* __restrict__ bi, BMap m) {
+__global__ void __launch_bounds__(kMaxSeqThreads + 32, sizeof(S) == 8 ? 4 : 1) k_bwd_seq_b(const BInst<S>* __restrict__ bi, BMap m) {
   const int i = m.inst[blockIdx.x], t = m.stage[i];
   const KP<S> p = bi[i].kp;
   bwd_seq_body<S, false>(p, t < 0 ? p.N : t, t < 0 ? p.chain_stage : t, blockIdx.x - m.base[i], m.cnt[i], 1);
 }
 template <typename S>
-__global__ void __launch_bounds__(kMaxSeqThreads + 32, 1) k_fwd_seq_b(const BInst<S>* __restrict__ bi, BMap m) {
+__global__ void __launch_bounds__(kMaxSeqThreads + 32, sizeof(S) == 8 ? 4 : 1) k_fwd_seq_b(const BInst<S>* __restrict__ bi, BMap m) {
   const int i = m.inst[blockIdx.x], t = m.stage[i];
   const KP<S> p = bi[i].kp;
   const int top = p.chain_stage > 0 ? p.chain_stage : 1;
@@ -533,16 +519,15 @@ static int num_sms() {
 }
 
 // Threads per block (without the fetching warp): a multiple of 32 that covers
-// the widest product, times row groups that shorten the serial sums.  Two row
-// groups where few sequences leave most of an SM to a block and the sums are
-// long enough to pay for the barrier between them (FP64, nx >= 12: 3.5 against
-// 4.0 us a backward step at nx = 50, nu = 20; FP32 1.36 against 1.31 us); one
-// where many blocks share an SM (FP64, 62,805 nodes: 670 us a backward chain
-// pass against 1,029 us).
-static int seq_threads(int nx, int nu, bool f64, bool many) {
-  const int CP = std::max(seq_cols(nx, nu), seq_cols(nu, nx));
-  const int rg = f64 && !many && nx >= 12 ? 2 : 1;
-  return std::min(kMaxSeqThreads / CP, rg) * CP;
+// the widest product times its row groups.  FP32 and FP64 below nx = 8: one
+// group (FP64, 3 to 6 states, 511 nodes: 92 to 94 us an evaluation of T with any
+// number; the groups' barriers cost what they save).
+template <typename S>
+static int seq_threads(int nx, int nu, int groups) {
+  const int CP = std::max(seq_cols<S>(nx, nu), seq_cols<S>(nu, nx));
+  if (sizeof(S) == 4) return CP;
+  const int rg = nx < 8 ? 1 : std::max(1, std::min(groups, kMaxSeqThreads / CP));
+  return (rg * CP + 31) & ~31;
 }
 
 struct SeqShape {
@@ -550,26 +535,40 @@ struct SeqShape {
   size_t bytes;
 };
 
-// Threads, slots and grid for `cnt` sequences of Lq nodes.  More than two
-// sequences per SM: one slot, and as many blocks as are resident -- at nx = 50,
-// nu = 20 four FP64 or eight FP32 ones, which hide one another's copies
-// better than a second slot does with half the blocks (FP64 chains of the
-// 62,805-node tree: 670 against 957 us).  Fewer: a second slot, if the
-// sequences are longer than one node and it fits.
+// Threads, slots and grid for `cnt` sequences of Lq nodes.
+//
+// Slots: more than two sequences per SM: one, and as many blocks as are resident
+// (at nx = 50, nu = 20 four FP64 or eight FP32 ones), which hide one another's
+// copies better than a second slot does with half the blocks (FP64 chains of the
+// 62,805-node tree: 670 against 957 us with integer products in their place).
+// Fewer: a second slot, if the sequences are longer than one node and it fits.
+//
+// FP64 row groups spread a node's multiply-adds over the four FP64 pipes of an
+// SM.  Few sequences: up to four (one evaluation of T on 511 nodes, one to four
+// groups: nx = 12, nu = 5 103, 92, 92, 92 us; 24, 12 117, 105, 103, 98; 50, 20
+// 156, 130, 122, 122).  Many, whose blocks fill the pipes together: two (4,437
+// nodes, one to three groups: 24, 12 149, 137, 147; 33, 15 182, 158, 171; 21,845
+// nodes: 33, 15 475, 440, 473); three where the nodes' size leaves shared memory
+// for five blocks or fewer (4,437 nodes, 50, 20: 273, 248, 225; 21,845 nodes:
+// 787, 720, 682; 64, 32: 329, 325, 324).
 template <typename S, typename F>
 static SeqShape seq_shape(const KP<S>& p, int cnt, int Lq, F layout) {
   SeqShape s;
   const int sms = num_sms();
   const bool many = cnt > 2 * sms;
-  s.T = seq_threads(p.nx, p.nu, sizeof(S) == 8, many);
-  const SeqLayout L = layout(p, s.T);
-  s.D = !many && Lq > 1 ? 2 : 1;
+  auto fit = [](size_t bytes) { return (int)(228 * 1024 / (bytes + 1280)); };   // static part and the 1 KB of the system
+  s.T = seq_threads<S>(p.nx, p.nu, many ? 2 : kMaxGroups);
+  SeqLayout L = layout(p, s.T);
+  if (sizeof(S) == 8 && many && fit(L.bytes(1)) < 6) {
+    s.T = seq_threads<S>(p.nx, p.nu, 3);
+    L = layout(p, s.T);
+  }
+  s.D = !many && Lq > 1 ? kMaxSlots : 1;
   while (s.D > 1 && L.bytes(s.D) > max_dyn_smem() - 512) --s.D;
   s.bytes = L.bytes(s.D);
-  const int by_smem = (int)(228 * 1024 / (s.bytes + 1280));   // static part and the 1 KB of the system
-  const int regs = sizeof(S) == 8 ? 112 : 80;
+  const int regs = sizeof(S) == 8 ? 64 : 80;
   const int by_thr = std::min(2048 / (s.T + 32), 65536 / ((s.T + 32) * regs));
-  const int blocks = std::max(1, std::min(32, std::min(by_smem, by_thr)));
+  const int blocks = std::max(1, std::min(32, std::min(fit(s.bytes), by_thr)));
   s.grid = std::max(1, std::min(cnt, sms * blocks));
   return s;
 }
@@ -610,12 +609,12 @@ int launch_fwd_seq(const KP<S>& p, int t_lo, int t_hi, int cnt, S* zo, cudaStrea
   return 1;
 }
 
-// One shape for a batch: the most threads and shared memory over the
-// instances.  Returns false if some instance's layout does not fit.
+// One shape for a batch, whose blocks fill the SMs together: the most threads and
+// shared memory over the instances.  Returns false if some instance's layout does not fit.
 template <typename S>
 bool seq_batch_shape(const std::vector<KP<S>>& kps, SeqBatchShape& sh) {
   sh.T = 32;
-  for (const KP<S>& p : kps) sh.T = std::max(sh.T, seq_threads(p.nx, p.nu, sizeof(S) == 8, true));
+  for (const KP<S>& p : kps) sh.T = std::max(sh.T, seq_threads<S>(p.nx, p.nu, 2));
   sh.bytes_bwd = sh.bytes_fwd = 0;
   for (const KP<S>& p : kps) {
     sh.bytes_bwd = std::max(sh.bytes_bwd, seq_layout_bwd(p, sh.T).bytes(1));

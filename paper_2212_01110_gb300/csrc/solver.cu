@@ -1793,18 +1793,16 @@ static int32_t pad16(int64_t elems, size_t elt) {
 enum BlockKind : int { BK_GB = 0, BK_NB = 1, BK_GF = 2, BK_KT = 3 };
 template <typename S>
 __global__ void k_factor_blocks(int kind, int nx, int nu, const double* __restrict__ in, int64_t stride,
-                                unsigned char* __restrict__ out, int64_t blockB, int64_t count) {
-  using Mat = typename Fx<S>::Mat;
+                                S* __restrict__ out, int64_t ostride, int64_t count) {
   const int ncol = nx + nu;
   const int nrow = kind == BK_GB ? nx : (kind == BK_NB ? 2 * nu : (kind == BK_GF ? ncol : nx));
   const int nc = kind == BK_GF ? nx : (kind == BK_KT ? nu : ncol);
-  const int64_t entries = kind == BK_NB ? (int64_t)nu * ncol + nu * nx : (int64_t)nrow * nc;
   const int64_t total = count * nc;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t b = i / nc;
     const int c = (int)(i % nc);
     const double* a = in + b * stride;
-    Mat* o = reinterpret_cast<Mat*>(out + b * blockB);
+    S* o = out + b * ostride;
     auto entry = [&](int r) -> double {
       if (kind == BK_GB) return a[(int64_t)r * ncol + (c < nu ? nx + c : c - nu)];
       if (kind == BK_GF) return a[(int64_t)c * ncol + r];
@@ -1821,20 +1819,7 @@ __global__ void k_factor_blocks(int kind, int nx, int nu, const double* __restri
       return kind == BK_NB && r >= nu ? (int64_t)nu * ncol + (int64_t)(r - nu) * nx + (c - nu) : (int64_t)r * nc + c;
     };
     const int nr = kind == BK_NB && c < nu ? nu : nrow;
-    if constexpr (sizeof(S) == 4) {
-      for (int r = 0; r < nr; ++r) o[place(r)] = (float)entry(r);
-    } else {
-      double big = 0.0;
-      for (int r = 0; r < nr; ++r) big = fmax(big, fabs(entry(r)));
-      // |entries| < 2^e; sums of more than 128 products get a bit of headroom
-      const int e = (big > 0.0 ? ilogb(big) + 1 : 0) + (nr > 128 ? 1 : 0);
-      reinterpret_cast<int32_t*>(o + entries)[c] = e;
-      for (int r = 0; r < nr; ++r) {
-        const long long v = llrint(scalbn(entry(r), 2 * kFxBits - e)), half = 1ll << (kFxBits - 1);
-        const int lo = (int)(((v + half) & ((1ll << kFxBits) - 1)) - half);
-        o[place(r)] = make_int2((int)((v - lo) >> kFxBits), lo);
-      }
-    }
+    for (int r = 0; r < nr; ++r) o[place(r)] = (S)entry(r);
   }
 }
 
@@ -1846,11 +1831,11 @@ static void factor_blocks(Problem& P, DevFactors<S>& f) {
   const int64_t n1 = P.tree.n - 1, nl = P.tree.n_nonleaf;
   auto build = [&](int kind, const double* in, int64_t stride, int64_t count, int64_t entries, int cols,
                    uint32_t& blockB) {
-    blockB = up128((uint32_t)(entries * sizeof(typename Fx<S>::Mat) + (sizeof(S) == 8 ? cols * sizeof(int32_t) : 0)));
-    unsigned char* b = dalloc<unsigned char>(P, (size_t)count * blockB);
+    blockB = up128((uint32_t)(entries * sizeof(S)));
+    S* b = dalloc<S>(P, (size_t)count * blockB / sizeof(S));
     CUDA_TRY(cudaMemsetAsync(b, 0, (size_t)count * blockB));   // the padding is copied along
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((count * cols + 127) / 128, (int64_t)sm_count() * 16));
-    k_factor_blocks<S><<<grid, 128>>>(kind, nx, nu, in, stride, b, blockB, count);
+    k_factor_blocks<S><<<grid, 128>>>(kind, nx, nu, in, stride, b, (int64_t)(blockB / sizeof(S)), count);
     check_launch();
     return b;
   };

@@ -59,7 +59,7 @@ struct DevFactors {
   S* NB = nullptr;   // [nl][K (nu x nx) | K + W^T (nu x nx) | Rtilde^-1 (nu x nu)]
   S* Kt = nullptr;   // [nl][nx][nu]      K^T
   // the factors in the blocks of the sequence kernels (KP in kernels.cuh)
-  unsigned char *pGb = nullptr, *pGf = nullptr, *pNB = nullptr, *pKt = nullptr;
+  S *pGb = nullptr, *pGf = nullptr, *pNB = nullptr, *pKt = nullptr;
   uint32_t gbB = 0, gfB = 0, nbB = 0, ktB = 0;
   S* qs = nullptr;   // [n][nx]  sqrt(Q) of the edge into the node
   S* rs = nullptr;   // [n][nu]  sqrt(R)
