@@ -199,4 +199,26 @@ bool riccati_factor(const Tree& t, int nx, int nu, const std::vector<double>& A,
   return ok;
 }
 
+void backward_blocks(int nx, int nu, std::vector<double>& NB, int threads) {
+  const size_t kx = (size_t)nu * nx, nbsz = 2 * kx + (size_t)nu * nu;
+  const int64_t nl = (int64_t)(NB.size() / nbsz);
+  const int nth = std::max(1, std::min(threads, (int)((nl + 63) / 64)));
+  auto work = [&](int tid) {
+    std::vector<double> E(kx);
+    for (int64_t k = tid; k < nl; k += nth) {
+      double* nb = &NB[(size_t)k * nbsz];
+      gemm(nu, nu, nx, nb + 2 * kx, nb + kx, E.data());
+      std::copy(nb, nb + kx, nb + kx);
+      std::copy(E.begin(), E.end(), nb);
+    }
+  };
+  if (nth == 1) {
+    work(0);
+    return;
+  }
+  std::vector<std::thread> pool;
+  for (int tid = 0; tid < nth; ++tid) pool.emplace_back(work, tid);
+  for (auto& th : pool) th.join();
+}
+
 }  // namespace spock

@@ -118,17 +118,7 @@ struct KP {
   const S* __restrict__ Gf;
   const S* __restrict__ NB;
   const S* __restrict__ Kt;
-  // the factors as the sequence kernels read them (riccati_seq.cu), per matrix
-  // one 128-byte aligned block of gbB, gfB, nbB, ktB bytes, row-major:
-  //   pGb  [B | Abar] (nx x (nu + nx)),  pGf  [Abar | B]^T ((nx + nu) x nx),
-  //   pNB  [Rtilde^-1 | E] (nu x (nu + nx)) and K (nu x nx), E = Rtilde^-1 (K + W^T),
-  //   pKt  K^T (nx x nu).
-  const S* __restrict__ pGb;
-  const S* __restrict__ pGf;
-  const S* __restrict__ pNB;
-  const S* __restrict__ pKt;
-  uint32_t gbB, gfB, nbB, ktB;
-  S* __restrict__ hb;   // [n - 1][hst] [B^c | Abar^c]^T q^c of the nonroot nodes
+  S* __restrict__ hb;   // [n - 1][hst] [Abar^c | B^c]^T q^c of the nonroot nodes
   int32_t hst;
   const S* __restrict__ qs;
   const S* __restrict__ rs;

@@ -6,7 +6,9 @@
 //   d^i = Rt^-1 (ubar^i - sum_c B^cT q^c)
 //   q^i = K^iT (d^i - ubar^i) - xbar^i + W^i d^i + sum_c Abar^cT q^c
 // (W^i = sum_c Abar^cT P^c B^c gathers the P^c B^c d^i terms of the paper's
-// recursion).  Forward pass from x^0 = x:
+// recursion); as read, q^i = E^iT g^i - K^iT ubar^i - xbar^i + sum_c Abar^cT q^c
+// with g^i = ubar^i - sum_c B^cT q^c and E = Rt^-1 (K + W^T).  Forward pass from
+// x^0 = x:
 //   u^i = K^i x^i + d^i,   x^c = A^c x^i + B^c u^i = Abar^c x^i + B^c d^i.
 //
 // GB300 mapping.  One warp owns one node at a time.  Every factor is read

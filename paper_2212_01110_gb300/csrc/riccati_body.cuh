@@ -51,9 +51,9 @@ __device__ __forceinline__ void node_bwd(const KP<S>& p, int k, const S (&h)[SL]
   __syncwarp();
   for (int b = lane; b < nu; b += 32) v.g[b] = v.u[b] - v.h[nx + b];
   __syncwarp();
-  const S* __restrict__ Km = p.NB + (int64_t)k * p.nbstride;
-  const S* __restrict__ Cm = Km + (int64_t)nu * nx;   // K + W^T
-  const S* __restrict__ Ri = Km + 2 * (int64_t)nu * nx;
+  const S* __restrict__ Em = p.NB + (int64_t)k * p.nbstride;   // Rtilde^-1 (K + W^T)
+  const S* __restrict__ Km = Em + (int64_t)nu * nx;
+  const S* __restrict__ Ri = Em + 2 * (int64_t)nu * nx;
   for (int a = lane; a < nu; a += 32) {
     S acc = 0;
     // Rtilde^-1 is stored exactly symmetric: lane a reads column a (row a),
@@ -70,17 +70,17 @@ __device__ __forceinline__ void node_bwd(const KP<S>& p, int k, const S (&h)[SL]
     const int r = 32 * s + lane;
     qn[s] = (r < nx) ? v.h[r] - xb[r] : S(0);
   }
-  // q += K^T (d - ubar) + W d = C^T d - K^T ubar
+  // q += K^T (d - ubar) + W d = E^T g - K^T ubar
 #pragma unroll 4
   for (int b = 0; b < nu; ++b) {
-    const S db = v.d[b];
+    const S gb = v.g[b];
     const S ub = v.u[b];
     const S* kr = Km + (int64_t)b * nx;
-    const S* cr = Cm + (int64_t)b * nx;
+    const S* er = Em + (int64_t)b * nx;
 #pragma unroll
     for (int s = 0; s < SL; ++s) {
       const int r = 32 * s + lane;
-      if (r < nx) qn[s] = fma(-__ldg(kr + r), ub, fma(__ldg(cr + r), db, qn[s]));   // two FMAs, no add
+      if (r < nx) qn[s] = fma(-__ldg(kr + r), ub, fma(__ldg(er + r), gb, qn[s]));   // two FMAs, no add
     }
   }
   __syncwarp();

@@ -10,8 +10,10 @@
 //   d^k = Rt^-1 g,   q^k = h_x - xbar^k + E^T g - K^T ubar^k
 //   h^k = [Abar^k | B^k]^T q^k                   (not at the root)
 // with E = Rt^-1 (K + W^T), formed once with the factors (q^k = h_x - xbar^k +
-// K^T (d^k - ubar^k) + W d^k, so that d^k and q^k come from one product), reads
-// the factors of node k only and hands nx + nu numbers on to the parent: in
+// K^T (d^k - ubar^k) + W d^k, so that d^k and q^k come from one product; K + W^T is
+// zero but for what rounding K left in Rt K, and taking it along keeps the
+// projection as exact as K allows: without it states in mixed units lose up to a
+// digit and a half), reads the factors of node k only and hands nx + nu numbers on to the parent: in
 // registers along a sequence, through p.hb between launches.  A branching
 // stage reads a quarter of what a step over the children's [Abar | B] reads at
 // four children per node; those of the chains' tops are streamed by the chain
@@ -34,7 +36,7 @@
 // differ by 1e6, 5e-4 by 1e12, against 2e-15.)
 //
 // What bounds it and what it measured (GB300, nx = 50, nu = 20).  Chains of the
-// 62,805-node tree, FP64: backward 837 us (2.75 GB), forward 611 us (2.2 GB),
+// 62,805-node tree, FP64: backward 853 us (2.75 GB), forward 606 us (2.2 GB),
 // where direct-load kernels took 1,073 and 705 us; the FP32 chains of 4,096
 // sequences of five nodes run at 5.2 - 5.6 TB/s.  The FP64 chains are bound by
 // the FP64 pipes (1.9 multiply-adds per clock and SM: a warp instruction holds
@@ -70,7 +72,7 @@ __host__ __device__ inline int up4(int n) { return (n + 3) & ~3; }
 template <typename S>
 __host__ __device__ inline SeqLayout seq_layout_bwd(const KP<S>& p, int T) {
   SeqLayout L;
-  L.item = up128(p.gbB + p.nbB + (p.xs + p.us) * (uint32_t)sizeof(S));   // [B | Abar] | node block | xbar | ubar
+  L.item = up128((p.gstride + p.nbstride + p.xs + p.us) * (uint32_t)sizeof(S));   // [Abar | B] | [E | K | Rt^-1] | xbar | ubar
   L.vecA = up16(2 * up4(p.nu) * (uint32_t)sizeof(S));                               // (g; -ubar)
   L.vecB = up16(up4(p.nx) * (uint32_t)sizeof(S));                                   // q
   L.part = up16(T * (uint32_t)sizeof(S));
@@ -79,7 +81,7 @@ __host__ __device__ inline SeqLayout seq_layout_bwd(const KP<S>& p, int T) {
 template <typename S>
 __host__ __device__ inline SeqLayout seq_layout_fwd(const KP<S>& p, int T) {
   SeqLayout L;
-  L.item = up128(p.gfB + p.ktB + p.us * (uint32_t)sizeof(S));   // [Abar | B]^T | K^T of the parent | d of the node
+  L.item = up128((p.gstride + p.ktstride + p.us) * (uint32_t)sizeof(S));   // [Abar | B]^T | K^T of the parent | d of the node
   L.vecA = up16(up4(p.nx + p.nu) * (uint32_t)sizeof(S));                   // (x; d) of the parent and of the node
   L.vecB = L.vecA;
   L.part = up16(T * (uint32_t)sizeof(S));
@@ -89,26 +91,52 @@ __host__ __device__ inline SeqLayout seq_layout_fwd(const KP<S>& p, int T) {
 // Barrier of the T working threads of a block.
 __device__ __forceinline__ void seq_bar(int T) { named_bar(1, T); }
 
-// Columns of a product: two blocks of n0 and n1, thread (row group, column).
-// FP32: the second block from a warp boundary on (both in one warp when they
-// fit), so that no warp runs the sums of both: with n0 = 50 and n1 = 20 packed
-// into 70 threads, one warp ran 120 rows where the others ran 70.  FP64: a warp
-// instruction holds its sub-partition's FP64 pipe for 64 cycles whatever its
-// lanes do, so the columns of all row groups are packed and few lanes idle
-// (nx = 50, nu = 20, three groups: 210 of 224 lanes).
+// Columns of a product: those of x (nx) and those of u (nu), a thread each, in
+// RG row groups.  FP32: per row group the x columns, then the u columns from a
+// warp boundary on (both in one warp when they fit), so that no warp runs the
+// sums of both: with 50 and 20 packed into 70 threads, one warp ran 120 rows
+// where the others ran 70.  FP64: a warp instruction holds its sub-partition's
+// FP64 pipe for 64 cycles whatever its lanes do, so the x columns of all row
+// groups come first, then the u columns, without gaps (nx = 50, nu = 20, three
+// groups: 210 of 224 lanes; few warps run the longer sums for columns of both).
 template <typename S>
-__host__ __device__ inline int seq_off(int n0, int n1) {
-  return sizeof(S) == 8 || n0 + n1 <= 32 ? n0 : (n0 + 31) & ~31;
-}
+__host__ __device__ inline int seq_off(int nx, int nu) { return nx + nu <= 32 ? nx : (nx + 31) & ~31; }
 template <typename S>
-__host__ __device__ inline int seq_cols(int n0, int n1) {
-  return sizeof(S) == 8 ? n0 + n1 : (seq_off<S>(n0, n1) + n1 + 31) & ~31;
+__host__ __device__ inline int seq_cols(int nx, int nu) {   // threads of one row group
+  return sizeof(S) == 8 ? nx + nu : (seq_off<S>(nx, nu) + nu + 31) & ~31;
 }
-// Row groups of a product of CP columns in T threads, and the rows of each.
+struct SeqCols {
+  int RG;       // row groups
+  int rg, col;  // this thread's group and its column of x or of u
+  int off;      // thread of the first u column of group 0
+  int step;     // threads from a column's group to its next group
+  bool xcol, live;
+};
 template <typename S>
-__device__ __forceinline__ int seq_groups(int T, int CP) {
-  return sizeof(S) == 8 ? min(T / CP, kMaxGroups) : T / CP;
+__device__ __forceinline__ SeqCols seq_columns(int nx, int nu, int T, int tid) {
+  SeqCols c;
+  const int CP = seq_cols<S>(nx, nu);
+  if (sizeof(S) == 8) {
+    c.RG = min(T / CP, kMaxGroups);
+    c.off = c.RG * nx;
+    c.xcol = tid < c.off;
+    c.step = c.xcol ? nx : nu;
+    const int t = c.xcol ? tid : tid - c.off;
+    c.rg = t / c.step;
+    c.col = t - c.rg * c.step;
+  } else {
+    c.RG = T / CP;
+    c.off = seq_off<S>(nx, nu);
+    c.step = CP;
+    c.rg = tid / CP;
+    const int t = tid - c.rg * CP;
+    c.xcol = t < nx;
+    c.col = c.xcol ? t : t - c.off;
+  }
+  c.live = c.rg < c.RG && c.col >= 0 && c.col < (c.xcol ? nx : nu);
+  return c;
 }
+// Rows of a row group.
 template <typename S>
 __device__ __forceinline__ int seq_chunk(int n, int RG) {
   const int c = (n + RG - 1) / RG;
@@ -158,16 +186,15 @@ __device__ __forceinline__ double seq_rows(double acc, uint32_t m, uint32_t ldB,
   return acc;
 }
 
-// Sum of the row groups' accumulators in the threads of row group 0, a column's
-// threads `step` apart (one barrier if there is more than one group; every
-// thread calls it).
+// Sum of the row groups' accumulators in the threads of row group 0 (one
+// barrier if there is more than one group; every thread calls it).
 template <typename S>
-__device__ __forceinline__ S seq_reduce(S acc, int rg, int RG, int step, bool live, S* part, int T) {
-  if (RG == 1) return acc;
-  if (live && rg > 0) part[threadIdx.x] = acc;
+__device__ __forceinline__ S seq_reduce(S acc, const SeqCols& c, bool live, S* part, int T) {
+  if (c.RG == 1) return acc;
+  if (live && c.rg > 0) part[threadIdx.x] = acc;
   seq_bar(T);
-  if (live && rg == 0)
-    for (int i = 1; i < RG; ++i) acc += part[i * step + threadIdx.x];
+  if (live && c.rg == 0)
+    for (int i = 1; i < c.RG; ++i) acc += part[i * c.step + threadIdx.x];
   return acc;
 }
 
@@ -242,6 +269,7 @@ __device__ __forceinline__ void bwd_seq_body(const KP<S>& p, int t_hi, int t_lo,
   __shared__ uint64_t bars[2][kMaxSlots];
   const int tid = threadIdx.x, T = blockDim.x - 32;
   const int nx = p.nx, nu = p.nu, ncol = nx + nu;
+  const uint32_t gB = p.gstride * B, nbB = p.nbstride * B;   // bytes of a node's blocks
   const SeqLayout Ly = seq_layout_bwd(p, T);
   const int cnt = p.stage_begin[t_lo + 1] - p.stage_begin[t_lo];
   if (bid >= cnt) return;
@@ -263,12 +291,12 @@ __device__ __forceinline__ void bwd_seq_body(const KP<S>& p, int t_hi, int t_lo,
           const bool leaf = k >= p.nl;
           unsigned char* dst = smem + slot * Ly.item;
           uint64_t* bar = &ring.full[slot];
-          mbar_expect_tx(bar, xB + (leaf ? 0u : p.nbB + uB) + (k > 0 ? p.gbB : 0u));
-          if (!leaf) bulk_g2s(dst + p.gbB, reinterpret_cast<const unsigned char*>(p.pNB) + (size_t)k * p.nbB, p.nbB, bar);
-          if (k > 0) bulk_g2s(dst, reinterpret_cast<const unsigned char*>(p.pGb) + (size_t)(k - 1) * p.gbB, p.gbB, bar);
+          mbar_expect_tx(bar, xB + (leaf ? 0u : nbB + uB) + (k > 0 ? gB : 0u));
+          if (!leaf) bulk_g2s(dst + gB, p.NB + (size_t)k * p.nbstride, nbB, bar);
+          if (k > 0) bulk_g2s(dst, p.Gb + (size_t)(k - 1) * p.gstride, gB, bar);
         },
         [&](int slot, int k, int) {
-          unsigned char* dst = smem + slot * Ly.item + p.gbB + p.nbB;
+          unsigned char* dst = smem + slot * Ly.item + gB + nbB;
           if (k < p.nl) bulk_g2s(dst + xB, p.ubar + (size_t)k * p.us, uB, &ring.full[slot]);
           bulk_g2s(dst, p.xbar + (size_t)k * p.xs, xB, &ring.full[slot]);
         });
@@ -280,16 +308,13 @@ __device__ __forceinline__ void bwd_seq_body(const KP<S>& p, int t_hi, int t_lo,
   S* const vB = reinterpret_cast<S*>(smem + D * Ly.item + Ly.vecA);     // q
   S* const part = reinterpret_cast<S*>(smem + D * Ly.item + Ly.vecA + Ly.vecB);
   const uint32_t aA = smem_u32(vA), aB = smem_u32(vB), a0 = smem_u32(smem);
-  // column col of row group rg: d and h_u in columns 0 .. nu - 1, q and h_x from
-  // column off on; mc the column in the matrices [.. (nu) | .. (nx)]; row group
-  // rg takes rows u0 .. or x0 .. of a vector
-  const int off = seq_off<S>(nu, nx), CP = seq_cols<S>(nu, nx), RG = seq_groups<S>(T, CP);
-  const int rg = tid / CP, col = tid - rg * CP;
-  const bool inu = tid < nu, inx = tid >= off && tid < off + nx, own = inu || inx;
-  const bool live = rg < RG && (col < nu || (col >= off && col < off + nx));
-  const int mc = col < nu ? col : col - off + nu, ex = tid - off;
-  const int nu4 = up4(nu), cu = seq_chunk<S>(nu, RG), cx = seq_chunk<S>(nx, RG);
-  const int u0 = rg * cu, un = max(0, min(cu, nu - u0)), x0 = rg * cx, xn = max(0, min(cx, nx - x0));
+  // q and h_x in the x columns, d and h_u in the u columns; entry e of h; row
+  // group rg takes rows u0 .. or x0 .. of a vector
+  const SeqCols cl = seq_columns<S>(nx, nu, T, tid);
+  const bool inx = tid < nx, inu = tid >= cl.off && tid < cl.off + nu, own = inx || inu;
+  const int a = tid - cl.off, e = inx ? tid : nx + a;
+  const int nu4 = up4(nu), cu = seq_chunk<S>(nu, cl.RG), cx = seq_chunk<S>(nx, cl.RG);
+  const int u0 = cl.rg * cu, un = max(0, min(cu, nu - u0)), x0 = cl.rg * cx, xn = max(0, min(cx, nx - x0));
   S h = S(0);   // h of the current node: this thread's column
   int slot = 0;
   for (int ci = bid; ci < cnt; ci += nblk) {
@@ -298,54 +323,56 @@ __device__ __forceinline__ void bwd_seq_body(const KP<S>& p, int t_hi, int t_lo,
       const bool leaf = k >= p.nl;
       if (t == t_hi && !leaf && own) {   // sum of the children's h, from the launch below
         const int c0 = p.ch_begin[k], m = p.ch_count[k];
-        const S* src = p.hb + (int64_t)(c0 - 1) * p.hst + mc;
+        const S* src = p.hb + (int64_t)(c0 - 1) * p.hst + e;
         h = src[0];
 #pragma unroll 4
         for (int c = 1; c < m; ++c) h += src[(int64_t)c * p.hst];
       }
       const unsigned char* it = smem + slot * Ly.item;
       const uint32_t ait = a0 + slot * Ly.item;
-      const S* xb = reinterpret_cast<const S*>(it + p.gbB + p.nbB);
+      const S* xb = reinterpret_cast<const S*>(it + gB + nbB);
       ring.wait(ring.full, slot, p.err);
       S q = S(0);
       if (leaf) {
-        if (inx) q = -xb[ex];
+        if (inx) q = -xb[tid];
       } else {
         if (inu) {
-          const S u = LAM ? h : (xb + p.xs)[tid];
-          vA[tid] = LAM ? S(0) : u - h;   // g
-          vA[nu4 + tid] = -u;
+          const S u = LAM ? h : (xb + p.xs)[a];
+          vA[a] = LAM ? S(0) : u - h;   // g
+          vA[nu4 + a] = -u;
         }
-        const S base = inx ? h - xb[ex] : S(0);
+        const S base = inx ? h - xb[tid] : S(0);
         seq_bar(T);
         S acc = S(0);
-        if (live) {   // [Rt^-1 | E] (nu x ncol), then K (nu x nx)
-          const uint32_t m1 = ait + p.gbB, m2 = m1 + nu * ncol * B;
-          acc = seq_rows(acc, m1 + (u0 * ncol + mc) * B, ncol * B, aA + u0 * B, un);
-          if (col >= off) acc = seq_rows(acc, m2 + (u0 * nx + mc - nu) * B, nx * B, aA + (nu4 + u0) * B, un);
+        if (cl.live) {   // E (nu x nx) or Rt^-1 (nu x nu) with g, then K (nu x nx) with -ubar
+          const uint32_t m = ait + gB;
+          acc = seq_rows(acc, m + (cl.xcol ? u0 * nx + cl.col : 2 * nu * nx + u0 * nu + cl.col) * B,
+                         (cl.xcol ? nx : nu) * B, aA + u0 * B, un);
+          if (cl.xcol) acc = seq_rows(acc, m + ((nu + u0) * nx + cl.col) * B, nx * B, aA + (nu4 + u0) * B, un);
         }
-        acc = seq_reduce<S>(acc, rg, RG, CP, live, part, T);
+        acc = seq_reduce<S>(acc, cl, cl.live, part, T);
         if (inx) q = base + acc;
         if (LAM) {
-          if (inx) lam[(int64_t)k * p.xs + ex] = q;
+          if (inx) lam[(int64_t)k * p.xs + tid] = q;
         } else if (inu) {
-          p.d[(int64_t)k * p.us + tid] = acc;
+          p.d[(int64_t)k * p.us + a] = acc;
         }
       }
       if (k > 0) {
-        if (inx) vB[ex] = q;
+        if (inx) vB[tid] = q;
         seq_bar(T);
         S acc = S(0);
-        if (live) acc = seq_rows(acc, ait + (x0 * ncol + mc) * B, ncol * B, aB + x0 * B, xn);
-        acc = seq_reduce<S>(acc, rg, RG, CP, live, part, T);
+        if (cl.live)   // [Abar | B] (nx x ncol)
+          acc = seq_rows(acc, ait + (x0 * ncol + (cl.xcol ? cl.col : nx + cl.col)) * B, ncol * B, aB + x0 * B, xn);
+        acc = seq_reduce<S>(acc, cl, cl.live, part, T);
         if (own) {
           h = acc;
-          if (t == t_lo) p.hb[(int64_t)(k - 1) * p.hst + mc] = h;
+          if (t == t_lo) p.hb[(int64_t)(k - 1) * p.hst + e] = h;
         }
         // every thread is through with the slot and the vectors; with several row
         // groups the barrier of the sum has said so (what group 0 reads after it,
         // the others' sums, is written again behind the next node's first barrier)
-        if (RG == 1) seq_bar(T);
+        if (cl.RG == 1) seq_bar(T);
         if (tid == 0) mbar_arrive(&ring.empty[slot]);
       }
       if (++slot == D) slot = 0;
@@ -362,6 +389,7 @@ __device__ __forceinline__ void fwd_seq_body(const KP<S>& p, int t_lo, int t_hi,
   __shared__ uint64_t bars[2][kMaxSlots];
   const int tid = threadIdx.x, T = blockDim.x - 32;
   const int nx = p.nx, nu = p.nu, ncol = nx + nu;
+  const uint32_t gB = p.gstride * B, ktB = p.ktstride * B;   // bytes of a node's blocks
   const SeqLayout Ly = seq_layout_fwd(p, T);
   const int cnt = p.stage_begin[t_lo + 1] - p.stage_begin[t_lo];
   if (bid >= cnt) return;
@@ -384,13 +412,13 @@ __device__ __forceinline__ void fwd_seq_body(const KP<S>& p, int t_lo, int t_hi,
           const bool first = above >= 0 || k == 1 || p.parent[k - 1] != par;   // k is its parent's first child
           unsigned char* dst = smem + slot * Ly.item;
           uint64_t* bar = &ring.full[slot];
-          mbar_expect_tx(bar, p.gfB + (first ? p.ktB : 0u) + (k < p.nl ? uB : 0u));
-          bulk_g2s(dst, reinterpret_cast<const unsigned char*>(p.pGf) + (size_t)(k - 1) * p.gfB, p.gfB, bar);
-          if (first) bulk_g2s(dst + p.gfB, reinterpret_cast<const unsigned char*>(p.pKt) + (size_t)par * p.ktB, p.ktB, bar);
+          mbar_expect_tx(bar, gB + (first ? ktB : 0u) + (k < p.nl ? uB : 0u));
+          bulk_g2s(dst, p.Gf + (size_t)(k - 1) * p.gstride, gB, bar);
+          if (first) bulk_g2s(dst + gB, p.Kt + (size_t)par * p.ktstride, ktB, bar);
         },
         [&](int slot, int k, int) {
           if (k < p.nl)
-            bulk_g2s(smem + slot * Ly.item + p.gfB + p.ktB, p.d + (size_t)k * p.us, uB, &ring.full[slot]);
+            bulk_g2s(smem + slot * Ly.item + gB + ktB, p.d + (size_t)k * p.us, uB, &ring.full[slot]);
         });
     return;
   }
@@ -400,21 +428,13 @@ __device__ __forceinline__ void fwd_seq_body(const KP<S>& p, int t_lo, int t_hi,
   S* Y = reinterpret_cast<S*>(smem + D * Ly.item + Ly.vecA);    // (x; d) of the node
   S* const part = reinterpret_cast<S*>(smem + D * Ly.item + Ly.vecA + Ly.vecB);
   const uint32_t a0 = smem_u32(smem);
-  // x (columns of ncol rows), then u of the parent (nx rows).  FP32: both in
-  // each row group.  FP64: the x columns of all groups first, so that few warps
-  // run the longer sums for columns of both (a step of the benchmark's tree:
-  // 154 warp instructions instead of 168).  The threads of row group 0 also
-  // hold the entries of (x; d), entry e.
-  const int CP = seq_cols<S>(nx, nu), RG = seq_groups<S>(T, CP);
-  const int off = sizeof(S) == 8 ? RG * nx : seq_off<S>(nx, nu);
-  const bool xcol = sizeof(S) == 8 ? tid < off : tid % CP < nx;
-  const int step = sizeof(S) == 4 ? CP : (xcol ? nx : nu);
-  const int rg = sizeof(S) == 4 ? tid / CP : (xcol ? tid / nx : (tid - off) / nu);
-  const int col = xcol ? tid - rg * step : tid - off - rg * step;   // of x or of u
-  const bool inx = tid < nx, inu = tid >= off && tid < off + nu, own = inx || inu;
-  const int a = tid - off, e = inx ? tid : nx + a;
-  const int cc = seq_chunk<S>(ncol, RG), cx = seq_chunk<S>(nx, RG);
-  const int w0 = rg * cc, wn = max(0, min(cc, ncol - w0)), x0 = rg * cx, xn = max(0, min(cx, nx - x0));
+  // x (ncol rows) and u of the parent (nx rows); the threads of row group 0 also
+  // hold the entries of (x; d), entry e
+  const SeqCols cl = seq_columns<S>(nx, nu, T, tid);
+  const bool inx = tid < nx, inu = tid >= cl.off && tid < cl.off + nu, own = inx || inu;
+  const int a = tid - cl.off, e = inx ? tid : nx + a;
+  const int cc = seq_chunk<S>(ncol, cl.RG), cx = seq_chunk<S>(nx, cl.RG);
+  const int w0 = cl.rg * cc, wn = max(0, min(cc, ncol - w0)), x0 = cl.rg * cx, xn = max(0, min(cx, nx - x0));
   S w = S(0);   // entry tid of the parent's (x; d)
   int slot = 0;
   for (int ci = bid; ci < cnt; ci += nblk) {
@@ -436,13 +456,12 @@ __device__ __forceinline__ void fwd_seq_body(const KP<S>& p, int t_lo, int t_hi,
       const unsigned char* it = smem + slot * Ly.item;
       const uint32_t ait = a0 + slot * Ly.item, aW = smem_u32(W);
       ring.wait(ring.full, slot, p.err);
-      const bool live = rg < RG && (xcol || (first && col >= 0 && col < nu));
+      const bool live = cl.live && (cl.xcol || first);
       S acc = S(0);
-      if (live) {   // [Abar | B]^T (ncol x nx) and K^T (nx x nu), one loop for both: a warp may hold columns of each
-        acc = seq_rows(acc, ait + (xcol ? (w0 * nx + col) * B : p.gfB + (x0 * nu + col) * B), (xcol ? nx : nu) * B,
-                       aW + (xcol ? w0 : x0) * B, xcol ? wn : xn);
-      }
-      acc = seq_reduce<S>(acc, rg, RG, step, live, part, T);
+      if (live)   // [Abar | B]^T (ncol x nx) or K^T (nx x nu), one loop: a warp may hold columns of both
+        acc = seq_rows(acc, ait + (cl.xcol ? (w0 * nx + cl.col) * B : gB + (x0 * nu + cl.col) * B),
+                       (cl.xcol ? nx : nu) * B, aW + (cl.xcol ? w0 : x0) * B, cl.xcol ? wn : xn);
+      acc = seq_reduce<S>(acc, cl, live, part, T);
       if (own && live) {
         if (inx) {
           zo[zxk + tid] = acc;
@@ -452,7 +471,7 @@ __device__ __forceinline__ void fwd_seq_body(const KP<S>& p, int t_lo, int t_hi,
         }
       }
       if (t < t_hi) {   // the node's (x; d) for the next step
-        if (inu) w = reinterpret_cast<const S*>(it + p.gfB + p.ktB)[a];
+        if (inu) w = reinterpret_cast<const S*>(it + gB + ktB)[a];
         if (own) Y[e] = w;
         S* y = W;
         W = Y;
@@ -524,7 +543,7 @@ static int num_sms() {
 // number; the groups' barriers cost what they save).
 template <typename S>
 static int seq_threads(int nx, int nu, int groups) {
-  const int CP = std::max(seq_cols<S>(nx, nu), seq_cols<S>(nu, nx));
+  const int CP = seq_cols<S>(nx, nu);
   if (sizeof(S) == 4) return CP;
   const int rg = nx < 8 ? 1 : std::max(1, std::min(groups, kMaxSeqThreads / CP));
   return (rg * CP + 31) & ~31;

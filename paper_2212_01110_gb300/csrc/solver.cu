@@ -316,14 +316,6 @@ static KP<S> make_kp(const Problem& P, double alpha, const int32_t* stage_begin_
   k.Gf = f.Gf;
   k.NB = f.NB;
   k.Kt = f.Kt;
-  k.pGb = f.pGb;
-  k.pGf = f.pGf;
-  k.pNB = f.pNB;
-  k.pKt = f.pKt;
-  k.gbB = f.gbB;
-  k.gfB = f.gfB;
-  k.nbB = f.nbB;
-  k.ktB = f.ktB;
   k.hb = f.hb;
   k.hst = f.hst;
   k.qs = f.qs;
@@ -1788,63 +1780,6 @@ static int32_t pad16(int64_t elems, size_t elt) {
   return (int32_t)((elems + a - 1) / a * a);
 }
 
-// One kind of factor block of the sequence kernels (KP in kernels.cuh), built
-// from the FP64 factors on the device: one thread per column of a block.
-enum BlockKind : int { BK_GB = 0, BK_NB = 1, BK_GF = 2, BK_KT = 3 };
-template <typename S>
-__global__ void k_factor_blocks(int kind, int nx, int nu, const double* __restrict__ in, int64_t stride,
-                                S* __restrict__ out, int64_t ostride, int64_t count) {
-  const int ncol = nx + nu;
-  const int nrow = kind == BK_GB ? nx : (kind == BK_NB ? 2 * nu : (kind == BK_GF ? ncol : nx));
-  const int nc = kind == BK_GF ? nx : (kind == BK_KT ? nu : ncol);
-  const int64_t total = count * nc;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t b = i / nc;
-    const int c = (int)(i % nc);
-    const double* a = in + b * stride;
-    S* o = out + b * ostride;
-    auto entry = [&](int r) -> double {
-      if (kind == BK_GB) return a[(int64_t)r * ncol + (c < nu ? nx + c : c - nu)];
-      if (kind == BK_GF) return a[(int64_t)c * ncol + r];
-      if (kind == BK_KT) return a[(int64_t)c * nx + r];
-      const double* C = a + (int64_t)nu * nx;         // K + W^T
-      const double* Ri = C + (int64_t)nu * nx;
-      if (r >= nu) return c < nu ? 0.0 : a[(int64_t)(r - nu) * nx + (c - nu)];
-      if (c < nu) return Ri[(int64_t)r * nu + c];
-      double e = 0.0;
-      for (int q = 0; q < nu; ++q) e = fma(Ri[(int64_t)r * nu + q], C[(int64_t)q * nx + (c - nu)], e);
-      return e;
-    };
-    auto place = [&](int r) -> int64_t {
-      return kind == BK_NB && r >= nu ? (int64_t)nu * ncol + (int64_t)(r - nu) * nx + (c - nu) : (int64_t)r * nc + c;
-    };
-    const int nr = kind == BK_NB && c < nu ? nu : nrow;
-    for (int r = 0; r < nr; ++r) o[place(r)] = (S)entry(r);
-  }
-}
-
-// Builds the blocks of precision S (the FP64 factors are on the device).
-template <typename S>
-static void factor_blocks(Problem& P, DevFactors<S>& f) {
-  const DevFactors<double>& src = P.f64;
-  const int nx = P.nx, nu = P.nu, ncol = nx + nu;
-  const int64_t n1 = P.tree.n - 1, nl = P.tree.n_nonleaf;
-  auto build = [&](int kind, const double* in, int64_t stride, int64_t count, int64_t entries, int cols,
-                   uint32_t& blockB) {
-    blockB = up128((uint32_t)(entries * sizeof(S)));
-    S* b = dalloc<S>(P, (size_t)count * blockB / sizeof(S));
-    CUDA_TRY(cudaMemsetAsync(b, 0, (size_t)count * blockB));   // the padding is copied along
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((count * cols + 127) / 128, (int64_t)sm_count() * 16));
-    k_factor_blocks<S><<<grid, 128>>>(kind, nx, nu, in, stride, b, (int64_t)(blockB / sizeof(S)), count);
-    check_launch();
-    return b;
-  };
-  f.pGb = build(BK_GB, src.Gb, src.gstride, n1, (int64_t)nx * ncol, ncol, f.gbB);
-  f.pGf = build(BK_GF, src.Gb, src.gstride, n1, (int64_t)nx * ncol, nx, f.gfB);
-  f.pNB = build(BK_NB, src.NB, src.nbstride, nl, (int64_t)nu * ncol + (int64_t)nu * nx, ncol, f.nbB);
-  f.pKt = build(BK_KT, src.NB, src.nbstride, nl, (int64_t)nx * nu, nu, f.ktB);
-}
-
 template <typename S>
 static void upload_factors(Problem& P, DevFactors<S>& f, const std::vector<double>& Gb,
                            const std::vector<double>& Gf, const std::vector<double>& NB,
@@ -1866,14 +1801,14 @@ static void upload_factors(Problem& P, DevFactors<S>& f, const std::vector<doubl
   const int nx = P.nx, nu = P.nu, ncol = nx + nu;
   f.xs = pad16(nx, sizeof(S));
   f.us = pad16(nu, sizeof(S));
-  f.gstride = pad16((int64_t)nx * ncol, sizeof(S));
-  f.nbstride = pad16(2 * (int64_t)nu * nx + (int64_t)nu * nu, sizeof(S));
-  f.ktstride = pad16((int64_t)nx * nu, sizeof(S));
+  auto pad128 = [](int64_t elems) { return (int32_t)(up128((uint32_t)(elems * sizeof(S))) / sizeof(S)); };
+  f.gstride = pad128((int64_t)nx * ncol);
+  f.nbstride = pad128(2 * (int64_t)nu * nx + (int64_t)nu * nu);
+  f.ktstride = pad128((int64_t)nx * nu);
   f.Gb = upload(P, padded(Gb, (size_t)nx * ncol, f.gstride));
   f.Gf = upload(P, padded(Gf, (size_t)nx * ncol, f.gstride));
   f.NB = upload(P, padded(NB, 2 * (size_t)nu * nx + (size_t)nu * nu, f.nbstride));
   f.Kt = upload(P, padded(Kt, (size_t)nx * nu, f.ktstride));
-  factor_blocks<S>(P, f);
   f.qs = upload(P, cast(par[0]));
   f.rs = upload(P, cast(par[1]));
   f.qns = upload(P, cast(par[2]));
@@ -2030,6 +1965,8 @@ static int problem_create(const Tree& tree, int32_t nx, int32_t nu, const double
       return fail(SPOCK_ERR_NUMERICAL, "Cholesky of I + sum B'PB failed");
     }
     P->factor_seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
+    // [K | K + W^T | Rtilde^-1] -> [E | K | Rtilde^-1]
+    backward_blocks(nx, nu, NB, threads);
     if (!all_finite(Gb.data(), Gb.size()) || !all_finite(NB.data(), NB.size())) {
       delete P;
       return fail(SPOCK_ERR_NUMERICAL, "non-finite Riccati factors");
@@ -2045,7 +1982,8 @@ static int problem_create(const Tree& tree, int32_t nx, int32_t nu, const double
     }
     for (int32_t k = 0; k < nl; ++k)
       for (int r = 0; r < nu; ++r)
-        for (int q = 0; q < nx; ++q) Kt[(size_t)k * nx * nu + (size_t)q * nu + r] = NB[(size_t)k * nbsz + (size_t)r * nx + q];
+        for (int q = 0; q < nx; ++q)
+          Kt[(size_t)k * nx * nu + (size_t)q * nu + r] = NB[(size_t)k * nbsz + (size_t)(nu + r) * nx + q];
     // node parameters (internal order)
     std::vector<std::vector<double>> par(9);
     par[0].assign(nn * nx, 0.0);

@@ -56,11 +56,8 @@ template <typename S>
 struct DevFactors {
   S* Gb = nullptr;   // [n-1][nx][nx+nu]  rows of [Abar^c | B^c], nonroot c
   S* Gf = nullptr;   // [n-1][nx+nu][nx]  transpose of the above
-  S* NB = nullptr;   // [nl][K (nu x nx) | K + W^T (nu x nx) | Rtilde^-1 (nu x nu)]
+  S* NB = nullptr;   // [nl][E (nu x nx) | K (nu x nx) | Rtilde^-1 (nu x nu)], E = Rtilde^-1 (K + W^T)
   S* Kt = nullptr;   // [nl][nx][nu]      K^T
-  // the factors in the blocks of the sequence kernels (KP in kernels.cuh)
-  S *pGb = nullptr, *pGf = nullptr, *pNB = nullptr, *pKt = nullptr;
-  uint32_t gbB = 0, gfB = 0, nbB = 0, ktB = 0;
   S* qs = nullptr;   // [n][nx]  sqrt(Q) of the edge into the node
   S* rs = nullptr;   // [n][nu]  sqrt(R)
   S* qns = nullptr;  // [n][nx]  sqrt(Q_N) (leaves)
@@ -92,7 +89,8 @@ struct DevFactors {
   S* x0 = nullptr;    // [nx]
   S* hb = nullptr;    // [n - 1][hst]
   int32_t hst = 0;
-  // per-node strides in elements, padded to a multiple of 16 bytes
+  // per-node strides in elements, padded to a multiple of 16 bytes (vectors) or of
+  // 128 (factors, which bulk copies fetch node by node)
   int32_t xs = 0, us = 0, gstride = 0, nbstride = 0, ktstride = 0;
 };
 
@@ -171,5 +169,8 @@ void build_offsets(const Tree& t, int nx, int nu, int nc, int ncN, const std::ve
 bool riccati_factor(const Tree& t, int nx, int nu, const std::vector<double>& A,
                     const std::vector<double>& B, std::vector<double>& Gb,
                     std::vector<double>& NB, int threads);
+// Each node's block of NB in the form that the backward step reads, in place:
+//   [E | K | Rtilde^-1],  E = Rtilde^-1 (K + W^T).
+void backward_blocks(int nx, int nu, std::vector<double>& NB, int threads);
 
 }  // namespace spock
