@@ -26,7 +26,6 @@
 // The backward layout [Abar^c | B^c] (nx x (nx+nu), row-major) serves
 // h = [Abar^c | B^c]^T q^c; the forward layout is its transpose so that
 // x^c = [Abar^c | B^c] (x; d) is again lanes-over-outputs.
-#include <cstdlib>
 
 #include "batch.cuh"
 #include "kernels.cuh"
@@ -67,10 +66,7 @@ int launch_fwd_seq(const KP<S>& p, int t_lo, int t_hi, int cnt, S* zo, cudaStrea
 // A single problem runs the staged sequence kernels; SPOCK_RICCATI_KERNELS =
 // direct forces the direct ones of this file (the tests cover both), which
 // the single-block solve and batches of very small problems use.
-static bool direct_kernels() {
-  const char* e = getenv("SPOCK_RICCATI_KERNELS");
-  return e && e[0] == 'd';
-}
+static bool direct_kernels() { return riccati_choice() == RK_DIRECT; }
 
 // Launches both passes; ev (optional, 3 events) is recorded after the
 // backward chain kernel, the backward stage kernels and the forward stage

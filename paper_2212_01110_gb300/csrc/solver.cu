@@ -747,9 +747,7 @@ static int solve_graph(Problem& P, const double* x0_dev, const spock_settings& s
     CUDA_TRY(cudaEventRecord(ws->e0, st));
     eval_T<S>(c, Vt, TVt, nullptr, stats_t, nullptr, false);  // T(v0); also sets kernel attributes outside capture
     const int64_t launches0 = ws->launches;
-    const char* fam = getenv("SPOCK_RICCATI_KERNELS");
-    const int trace_key = (trace_dev ? 1 : 0) + 2 * (s.profile ? 1 : 0) +
-                          4 * (fam && fam[0] ? (int)(unsigned char)fam[0] : 0);
+    const int trace_key = (trace_dev ? 1 : 0) + 2 * (s.profile ? 1 : 0) + 4 * (int)riccati_choice();
     if (s.profile) ws->prof.start();  // event slot r is recorded by round r of every replay
     if (!ws->gexec || ws->g_alpha != alpha || ws->g_trace != trace_key) {
       if (ws->gexec) {
@@ -997,8 +995,8 @@ __global__ void k_gather_done(SmState* const* __restrict__ sts, int n, int32_t* 
 // warp of the node kernels (the autotuned tile shape); the vector kernels
 // take kVecElemsPerThread elements per thread; the Riccati passes use the
 // direct kernels (fam 0: one warp per chain / node) or the staged ones
-// (fam 1: chain blocks of wpb warps, one block per branching node; falls
-// back to direct if a layout does not fit).
+// (fam 1: one block per node sequence, that is per chain or branching node;
+// falls back to direct if a layout does not fit).
 template <typename S>
 static void batch_plan(Batch& B, const std::vector<Workspace*>& wss, const std::vector<double>& alphas, int mem,
                        int tile, int fam) {
@@ -1248,8 +1246,8 @@ static void batch_init(Batch& B, const std::vector<Workspace*>& wss, const std::
 // single-block persistent solve (cta.cu).  Each candidate runs the
 // evaluation of T at the starting points and kTuneRounds rounds from the
 // same state; the fastest is cached per batch and precision.
-// SPOCK_BATCH_TILE fixes the tile, SPOCK_RICCATI_KERNELS the family (direct,
-// any other value: staged), SPOCK_BATCH_MODE = list / cta the mode.
+// SPOCK_BATCH_TILE fixes the tile, SPOCK_RICCATI_KERNELS the family
+// (riccati_choice), SPOCK_BATCH_MODE = list / cta the mode.
 constexpr int kTuneRounds = 4;
 struct BatchCfg {
   int tile, fam;
@@ -1285,9 +1283,9 @@ static BatchCfg batch_tune(Batch& B, const std::vector<Workspace*>& wss, const s
     const int t = atoi(env);
     if (t == 1 || t == 2 || t == 4 || t == 8 || t == 16) tiles = {t};
   }
-  const char* ek = getenv("SPOCK_RICCATI_KERNELS");
-  if (ek && ek[0] == 'd') fams = {0};
-  if (ek && ek[0] == 't') fams = {1};
+  const RiccatiChoice rk = riccati_choice();
+  if (rk == RK_DIRECT) fams = {0};
+  if (rk == RK_STAGED) fams = {1};
   bool cta_ok = true;
   for (const Problem* P : B.probs) cta_ok = cta_ok && cta_supported(P->nx, P->nu, mem);
   bool try_list = true;

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cstdint>
+#include <cstdlib>
 #include <string>
 #include <vector>
 
@@ -22,6 +23,17 @@ struct Error {
   int code;
   std::string msg;
 };
+
+// Riccati kernels that SPOCK_RICCATI_KERNELS asks for, of single problems and of
+// batches alike: unset, empty or "auto" leaves the choice to the library (single
+// problems: staged; batches: timed), "direct" (or d...) asks for the direct
+// kernels, any other value for the staged ones.  v: the variable's value.
+enum RiccatiChoice { RK_AUTO = 0, RK_DIRECT = 1, RK_STAGED = 2 };
+inline RiccatiChoice riccati_choice(const char* v) {
+  if (!v || !v[0] || std::string(v) == "auto") return RK_AUTO;
+  return v[0] == 'd' ? RK_DIRECT : RK_STAGED;
+}
+inline RiccatiChoice riccati_choice() { return riccati_choice(std::getenv("SPOCK_RICCATI_KERNELS")); }
 
 void set_error(const std::string& msg);
 int fail(int code, const std::string& msg);
