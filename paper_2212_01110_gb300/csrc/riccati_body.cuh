@@ -16,7 +16,6 @@ struct WarpVecs {
   S* h;  // [nx+nu]  accumulated [Abar | B]^T q over the children
   S* u;  // [nu]     ubar of the node
   S* g;  // [nu]     ubar - sum B^T q
-  S* d;  // [nu]
   S* w;  // [nx+nu]  forward input (x; d)
 };
 
@@ -59,10 +58,8 @@ __device__ __forceinline__ void node_bwd(const KP<S>& p, int k, const S (&h)[SL]
     // Rtilde^-1 is stored exactly symmetric: lane a reads column a (row a),
     // consecutive lanes consecutive addresses
     for (int b = 0; b < nu; ++b) acc += __ldg(Ri + b * nu + a) * v.g[b];
-    v.d[a] = acc;
     p.d[(int64_t)k * p.us + a] = acc;
   }
-  __syncwarp();
   S qn[SL];
   const S* xb = p.xbar + (int64_t)k * p.xs;
 #pragma unroll
@@ -135,10 +132,9 @@ __device__ __forceinline__ void child_fwd(const S* __restrict__ Gf, const S* w, 
   __shared__ S sm_h[kWarpsPerBlock][kVP_];                           \
   __shared__ S sm_u[kWarpsPerBlock][kVP_];                           \
   __shared__ S sm_g[kWarpsPerBlock][kVP_];                           \
-  __shared__ S sm_d[kWarpsPerBlock][kVP_];                           \
   __shared__ S sm_w[kWarpsPerBlock][kVP_];                           \
   const int wl_ = threadIdx.x >> 5;                                  \
-  WarpVecs<S> v{sm_q[wl_], sm_h[wl_], sm_u[wl_], sm_g[wl_], sm_d[wl_], sm_w[wl_]};
+  WarpVecs<S> v{sm_q[wl_], sm_h[wl_], sm_u[wl_], sm_g[wl_], sm_w[wl_]};
 
 // ---------------------------------------------------------------------------
 // backward, chain region: warp per chain, leaves up to the chain stage
