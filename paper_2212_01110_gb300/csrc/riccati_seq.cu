@@ -36,11 +36,12 @@
 // differ by 1e6, 5e-4 by 1e12, against 2e-15.)
 //
 // What bounds it and what it measured (GB300, nx = 50, nu = 20).  Chains of the
-// 62,805-node tree, FP64: backward 853 us (2.75 GB), forward 606 us (2.2 GB),
-// where direct-load kernels took 1,073 and 705 us; the FP32 chains of 4,096
-// sequences of five nodes run at 5.2 - 5.6 TB/s.  The FP64 chains are bound by
+// 62,805-node tree, FP64: backward 886 us (2.88 GB), forward 576 us (2.2 GB),
+// where direct-load kernels took 1,073 and 705 us; FP32: 228 and 174 us, 6.0 TB/s
+// (278 and 237 with one warp per chain).  The FP64 chains are bound by
 // the FP64 pipes (1.9 multiply-adds per clock and SM: a warp instruction holds
-// its sub-partition's pipe for 64 cycles), the FP32 ones by memory latency.
+// its sub-partition's pipe for 64 cycles; 85 and 88% busy), the FP32 ones by
+// memory.
 //
 // Bounded waits: a wait that exceeds kWaitLimit polls sets *p.err and the
 // thread stops waiting (the fetching warp: stops issuing); the block finishes
@@ -538,9 +539,10 @@ static int num_sms() {
 }
 
 // Threads per block (without the fetching warp): a multiple of 32 that covers
-// the widest product times its row groups.  FP32 and FP64 below nx = 8: one
-// group (FP64, 3 to 6 states, 511 nodes: 92 to 94 us an evaluation of T with any
-// number; the groups' barriers cost what they save).
+// the widest product times its row groups.  FP32 and FP64 below nx = 8: those of
+// one group (FP64, 3 to 6 states, 511 nodes: 92 to 94 us an evaluation of T with
+// any number; the groups' barriers cost what they save; a warp that holds several
+// groups of so few columns works in them all the same).
 template <typename S>
 static int seq_threads(int nx, int nu, int groups) {
   const int CP = seq_cols<S>(nx, nu);
@@ -556,11 +558,25 @@ struct SeqShape {
 
 // Threads, slots and grid for `cnt` sequences of Lq nodes.
 //
-// Slots: more than two sequences per SM: one, and as many blocks as are resident
-// (at nx = 50, nu = 20 four FP64 or eight FP32 ones), which hide one another's
-// copies better than a second slot does with half the blocks (FP64 chains of the
-// 62,805-node tree: 670 against 957 us with integer products in their place).
-// Fewer: a second slot, if the sequences are longer than one node and it fits.
+// Slots: two where they fit, so that a block fetches a node while it works on
+// the one before; half as many blocks are resident where shared memory bounds
+// them.  One after another the FP64 chain kernels take as long with one slot as
+// with two (62,805 nodes: 853 and 602 us, 884 and 575); in the stream, where a
+// launch's first blocks start beside the last of the one before, they do not.
+// One evaluation of T, one slot and two, us (nx, nu; nodes; chains):
+//   FP64  6, 3    8,533 1,024  112, 108      33, 15    661    64   92,  84
+//         24, 12    661    64   76,  69      33, 15 17,749 4,096  533, 371
+//         24, 12 17,749 4,096  447, 441      50, 20 17,749 4,096  724, 607
+//         64, 32 17,749 4,096 1,049, 985     50, 20 62,805 4,096 2,393, 2,017
+//   FP32  24, 12 17,749 4,096  126, 109      50, 20 62,805 4,096  618, 604
+// Sequences of one node gain by it only if blocks take several and a copy is
+// long: full binary tree of 4,095 nodes, FP64, 3 KB a node (12, 5) 121, 128; 13 KB
+// (24, 12) 178, 178; 48 KB (50, 20) 267, 240; a solve on 2,047 nodes, 16.5 KB (20,
+// 20) 1,747, 1,778: FP64 from 20 KB.  FP32 (from 16 KB) waits for memory and not for the
+// FP64 pipes and needs the blocks: with one block per SM many sequences lose
+// (90, 38, 17,749 nodes: 447, 476), with two the single nodes (a solve on a full
+// binary tree of 4,095 nodes, 50, 50: 1,396, 1,446; with four, on 21,845 nodes,
+// 50, 20, 18 and 24 KB a node: 2,445, 2,369).
 //
 // FP64 row groups spread a node's multiply-adds over the four FP64 pipes of an
 // SM.  Few sequences: up to four (one evaluation of T on 511 nodes, one to four
@@ -582,8 +598,9 @@ static SeqShape seq_shape(const KP<S>& p, int cnt, int Lq, F layout) {
     s.T = seq_threads<S>(p.nx, p.nu, 3);
     L = layout(p, s.T);
   }
-  s.D = !many && Lq > 1 ? kMaxSlots : 1;
-  while (s.D > 1 && L.bytes(s.D) > max_dyn_smem() - 512) --s.D;
+  s.D = Lq > 1 || (cnt > sms && L.item >= (sizeof(S) == 8 ? 20 : 16) * 1024) ? kMaxSlots : 1;
+  const int least = sizeof(S) == 8 ? 1 : (Lq == 1 ? 4 : (many ? 2 : 1));   // resident blocks
+  while (s.D > 1 && (L.bytes(s.D) > max_dyn_smem() - 512 || fit(L.bytes(s.D)) < least)) --s.D;
   s.bytes = L.bytes(s.D);
   const int regs = sizeof(S) == 8 ? 64 : 80;
   const int by_thr = std::min(2048 / (s.T + 32), 65536 / ((s.T + 32) * regs));
@@ -592,7 +609,11 @@ static SeqShape seq_shape(const KP<S>& p, int cnt, int Lq, F layout) {
   return s;
 }
 
-// Raises a kernel's dynamic shared-memory limit, once per kernel and device.
+// Raises a kernel's dynamic shared-memory limit, once per kernel and device, and
+// asks for the largest shared-memory carve-out: left to itself the driver chose
+// one per launch that held fewer blocks than planned (256 chains of nine nodes,
+// nx = 33, nu = 15, FP64, two slots: an evaluation of T took 139 us, 114 with it;
+// 64 chains of ten, 24, 12: 88, 69; FP32 within 3% either way).
 template <typename F>
 static void allow_smem(F* fn, std::atomic<uint64_t>& done) {
   int dev = 0;
@@ -600,6 +621,7 @@ static void allow_smem(F* fn, std::atomic<uint64_t>& done) {
   const uint64_t bit = 1ull << (dev & 63);
   if (done.load(std::memory_order_acquire) & bit) return;
   cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(max_dyn_smem() - 512));
+  cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   done.fetch_or(bit, std::memory_order_release);
 }
 
