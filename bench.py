@@ -45,16 +45,14 @@ def measured_peaks():
         return {}
 
 
-# DRAM bytes (read + write) per chain node of one launch of the backward
-# chain kernel (k_bwd_seq<double> / k_bwd_seq<float>), from ncu
-# captures on the 17,749-node tree (branching 4 for 6 stages, N = 9: 4,096
-# chains of 3 nonleaf nodes, nx = 50, nu = 20), scaled by the chain nodes of
-# the measured tree (each chain node's factors are read once).  Valid for the
-# kernels as captured (None: not captured since the kernel last changed);
-# remeasure after changing them.
-NCU_TRAFFIC_PER_CHAIN_NODE = {"fp64": None, "fp32": None}
+# DRAM bytes (read + write) of one launch of the backward chain kernel
+# (k_bwd_seq<double> / k_bwd_seq<float>) over the bytes it moves by its own
+# account (moved_bwd_chain), from ncu captures on the 17,749-node tree
+# (branching 4 for 6 stages, N = 9: 4,096 chains of 3 nonleaf nodes, nx = 50,
+# nu = 20).  Valid for the kernels as captured (None: not captured since the
+# kernel last changed); remeasure after changing them.
+NCU_TRAFFIC_RATIO = {"fp64": 710.319616e6 / 707.461120e6, "fp32": 357.954816e6 / 353.730560e6}
 NCU_CHAIN_SHAPE = (50, 20)   # nx, nu of the capture
-
 
 
 def replica_reduce(ms, units, dev=None):
@@ -124,12 +122,21 @@ class Clocks:
 
 def bytes_bwd_chain(d, n_chains, chain_len, elt):
     """Algorithmic bytes of one launch of the Riccati backward chain kernel:
-    per chain node [Abar|B] (nx (nx+nu)), K, W^T (2 nu nx), Rt^-1 (nu^2),
-    xbar and ubar reads (nx + nu), d write (nu); per chain the leaf's xbar
-    (nx) and the q of its top node (nx)."""
+    per chain node [Abar|B] (nx (nx+nu)), two nu x nx matrices (K and W^T as
+    Algorithm 2 has them, E and K here), Rt^-1 (nu^2), xbar and ubar reads
+    (nx + nu), d write (nu); per chain the leaf's xbar (nx) and the q of its
+    top node (nx)."""
     nx, nu = d["nx"], d["nu"]
     per_node = nx * (nx + nu) + 2 * nu * nx + nu * nu + nx + 2 * nu
     return elt * (n_chains * chain_len * per_node + n_chains * 2 * nx)
+
+
+def moved_bwd_chain(d, n_chains, chain_len, elt):
+    """Bytes that the launch moves: the algorithmic ones, with [Abar|B] of the
+    chain's top node, whose product is handed on in its place, and h (nx + nu)
+    instead of q."""
+    nx, nu = d["nx"], d["nu"]
+    return bytes_bwd_chain(d, n_chains, chain_len, elt) + elt * n_chains * (nx * (nx + nu) + nu)
 
 
 def flops_bwd_chain(d, n_chains, chain_len):
@@ -196,10 +203,10 @@ def run_ours(args, rank, world, local_rank):
         return ms, nT, nT_all, infos, clk.summary()
 
     def traffic(prec):
-        per = NCU_TRAFFIC_PER_CHAIN_NODE["fp64" if prec == spock.SPOCK_FP64 else "fp32"]
-        if per is None or (d["nx"], d["nu"]) != NCU_CHAIN_SHAPE:
+        ratio = NCU_TRAFFIC_RATIO["fp64" if prec == spock.SPOCK_FP64 else "fp32"]
+        if ratio is None or (d["nx"], d["nu"]) != NCU_CHAIN_SHAPE:
             return None
-        return round(per * n_chains * chain_len)
+        return round(ratio * moved_bwd_chain(d, n_chains, chain_len, 8 if prec == spock.SPOCK_FP64 else 4))
 
     def roofline(infos, prec):
         elt = 8 if prec == spock.SPOCK_FP64 else 4
@@ -210,17 +217,17 @@ def run_ours(args, rank, world, local_rank):
         fl = flops_bwd_chain(d, n_chains, chain_len)
         groups = {g: sum(i.t_group_ms[k] for i in infos) / max(timed_T, 1)
                   for k, g in enumerate(spock.Info.GROUPS)}
-        # both precisions against the bandwidth: the FP64 products are integer
-        # sums and not bound by the FP64 pipe (its rate beside them)
         ach = bb / (t_bwd * 1e-3) / 1e9
-        r = {"kernel": "k_bwd_seq<double>" if prec == spock.SPOCK_FP64 else "k_bwd_seq<float>", "bound": "hbm",
-             "achieved": round(ach, 1), "peak": hbm, "unit": "GB/s", "frac": round(ach / hbm, 4),
-             "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)",
-             "traffic": traffic(prec), "algorithmic_bytes": bb, "avg_launch_ms": round(t_bwd, 4)}
+        r = {"kernel": "k_bwd_seq<float>", "bound": "hbm", "achieved": round(ach, 1), "peak": hbm, "unit": "GB/s",
+             "frac": round(ach / hbm, 4), "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)"}
         if prec == spock.SPOCK_FP64:
             tf = fl / (t_bwd * 1e-3) / 1e12
-            r.update(algorithmic_flops=fl, achieved_tflops=round(tf, 4), fp64_fma_peak_tflops=round(fp64_peak, 4),
-                     frac_of_fp64_fma_peak=round(tf / fp64_peak, 4))
+            r = {"kernel": "k_bwd_seq<double>", "bound": "alu", "achieved": round(tf, 4),
+                 "peak": round(fp64_peak, 4), "unit": "TFLOP/s", "frac": round(tf / fp64_peak, 4),
+                 "peak_source": "measured in this run by spock_fp64_fma_rate (FP64 FMA throughput kernels, "
+                                "best over 8 / 16 chains per thread and 4 / 8 blocks per SM, best of 2 calls)",
+                 "algorithmic_flops": fl, "hbm_achieved_gbs": round(ach, 1), "hbm_frac_of_measured": round(ach / hbm, 4)}
+        r.update(traffic=traffic(prec), algorithmic_bytes=bb, avg_launch_ms=round(t_bwd, 4))
         fb = bytes_fwd_chain(d, n_chains, chain_len, elt)
         r["fwd_chain"] = {"avg_launch_ms": round(t_fwd, 4), "algorithmic_bytes": fb,
                           "achieved_gbs": round(fb / (t_fwd * 1e-3) / 1e9, 1) if t_fwd > 0 else None}
